@@ -523,7 +523,7 @@ def bench_batched(dev, stream, count=4096, seed=7, replays=20, warmup=3):
         torch.cuda.synchronize(dev)
         plain_ms.append(a.elapsed_time(b))
     pm = statistics.median(plain_ms)
-    out["plain_launches"] = {"launches": sum(p.num_passes for p in plans),
+    out["plain_launches"] = {"launches": sum(p.num_launches for p in plans),
                              "gbs": round(moved / (pm / 1e3) / 1e9, 1),
                              "ms": round(pm, 3)}
     out["speedup_vs_plain"] = round(pm / med, 3)
@@ -651,7 +651,7 @@ def bench_n20(dev, reps=50):
                      "gbs": round(2 * (1 << n) * 4 / (ms / 1e3) / 1e9, 1),
                      "graph_us_per_permutation": round(gms * 1e3, 2),
                      "graph_gbs": round(2 * (1 << n) * 4 / (gms / 1e3) / 1e9, 1),
-                     "launches": sum(p.num_passes for p in plans)}
+                     "launches": sum(p.num_launches for p in plans)}
         del graph
     return out
 
@@ -750,13 +750,13 @@ def bench_serving(dev, seconds=10.0, rate=2000.0, seed=11, budget=40 * 10**9, st
            "budget_bytes": budget, "streams": streams, "strategy": "paper",
            "server_large_log2": 28}
     # The latency floor with no queueing: each request's HBM traffic (2 N e
-    # per pass) at the measured peak; its 99th percentile bounds p99 from
+    # per launch) at the measured peak; its 99th percentile bounds p99 from
     # below at a rate that never queues.
     peak, _ = measured_hbm_peak()
     ideal = []
     for s_, (rows, c) in zip(specs, mats):
-        passes = bm.Plan(s_["n"], rows, c, s_["e"]).num_passes
-        ideal.append(passes * 2 * (1 << s_["n"]) * s_["e"] / (peak * 1e9) * 1e3)
+        launches = bm.Plan(s_["n"], rows, c, s_["e"]).num_launches
+        ideal.append(launches * 2 * (1 << s_["n"]) * s_["e"] / (peak * 1e9) * 1e3)
     res["ideal_service_ms"] = {"p50": round(_percentile(ideal, 0.5), 4),
                                "p99": round(_percentile(ideal, 0.99), 4),
                                "max": round(max(ideal), 4),
@@ -859,7 +859,7 @@ def main():
     bytes_per_step = sum(2 * N * e for (_, e, _, _) in items)
     total_bytes = allreduce_sum(world, float(bytes_per_step * K))
     value = total_bytes / (elapsed_ms / 1e3) / 1e9
-    launches_per_step = sum(p.num_passes for p in plans)
+    launches_per_step = sum(p.num_launches for p in plans)
 
     # per class / element size; per kernel instantiation (one per elem size)
     durs = [0.0] * len(items)
@@ -882,7 +882,7 @@ def main():
         key = "%s_e%d" % (cls, e)
         b = 2 * N * e
         d = by_class.setdefault(key, {"bytes": 0, "ms": 0.0, "count": 0,
-                                      "passes": plans[i].num_passes})
+                                      "launches": plans[i].num_launches})
         d["bytes"] += b
         d["ms"] += durs[i]
         d["count"] += 1
@@ -892,8 +892,8 @@ def main():
         kname = "%s<%d>" % ("bmmc_tiled_pass_tma" if args.load == "tma" else "bmmc_tiled_pass",
                             {4: 2, 8: 3, 16: 4}[e])
         kernel_time[kname] = kernel_time.get(kname, 0.0) + durs[i]
-        kernel_launches[kname] = kernel_launches.get(kname, 0) + plans[i].num_passes
-        kernel_bytes[kname] = kernel_bytes.get(kname, 0) + b * plans[i].num_passes
+        kernel_launches[kname] = kernel_launches.get(kname, 0) + plans[i].num_launches
+        kernel_bytes[kname] = kernel_bytes.get(kname, 0) + b * plans[i].num_launches
 
     # ---- same-run D2D copy baseline ---------------------------------------
     d2d = {}
@@ -915,7 +915,7 @@ def main():
         e = int(key.rsplit("_e", 1)[1])
         gbs = d["bytes"] / (statistics.median(class_steps[key]) / 1e3) / 1e9
         breakdown[key] = {"gbs": round(gbs, 1), "frac_of_d2d": round(gbs / d2d[e], 4),
-                          "passes": d["passes"], "count": d["count"]}
+                          "launches": d["launches"], "count": d["count"]}
 
     # ---- roofline of the dominant kernel ----------------------------------
     dom = max(kernel_time, key=kernel_time.get)

@@ -68,8 +68,10 @@ enum bmmc_status {
 /* Planning strategies (bmmc_plan_options.flags). */
 enum bmmc_plan_flags {
     /* The paper's method: a tiled BMMC (Sec. 5.1) runs as one pass; any other
-     * BMMC is factorised as A = (U R)(R L P) and runs as two tiled passes,
-     * (R L P, 0) first and then (U R, c) (Sec. 5.2). */
+     * BMMC is factorised as A = (U R)(R L P) into two tiled passes, (R L P, 0)
+     * first and then (U R, c) (Sec. 5.2).  The two are run as one launch over
+     * the tiles described below where these exist (always with the default
+     * segments): half the traffic, the same bytes. */
     BMMC_PLAN_PAPER = 0,
     /* One pass for every BMMC.  Each tile is a coset of the subspace spanned
      * by the low index bits and the kernel of the high output rows of A, so it
@@ -127,9 +129,13 @@ int bmmc_plan_create_ex(bmmc_plan *out, int n, const uint64_t *A_rows,
  * running. */
 void bmmc_plan_destroy(bmmc_plan p);
 
-/* Number of kernel passes bmmc_execute runs: 1 or 2 (Sec. 5.2).
+/* Number of tiled passes of the plan: 1 or 2 (Sec. 5.2).
  * Returns a negative code for a NULL plan. */
 int bmmc_plan_num_passes(bmmc_plan p);
+
+/* Number of kernel launches one execution makes: 1, also for a two-pass plan
+ * whose passes run fused, or 2.  Returns a negative code for a NULL plan. */
+int bmmc_plan_num_launches(bmmc_plan p);
 
 /* The plan's own matrix A (n row masks into rows_out) and complement c.
  * Errors: INVALID. */
@@ -184,9 +190,9 @@ size_t bmmc_plan_workspace_bytes(bmmc_plan p);
  * in, out  device buffers of 2^n * elem_bytes bytes (see conventions).
  * stream   CUDA stream to run on.
  *
- * A two-pass plan needs a workspace of bmmc_plan_workspace_bytes bytes; on
- * its first two-pass execution the plan allocates one (cudaMalloc) and keeps
- * it until bmmc_plan_destroy.  Because that workspace is shared, at most one
+ * A two-pass plan has a workspace of bmmc_plan_workspace_bytes bytes; on
+ * its first execution here the plan allocates one (cudaMalloc) and keeps
+ * it until bmmc_plan_destroy (bmmc_execute_direct needs none).  Because that workspace is shared, at most one
  * execution of a given plan may be in flight at a time with this entry
  * point; use bmmc_execute_ws with distinct workspaces for concurrent
  * executions of one plan.
@@ -200,6 +206,12 @@ int bmmc_execute(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream);
  * Errors: INVALID, ALIAS, ALIGN, CUDA. */
 int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws,
                     bmmc_stream_t stream);
+
+/* As bmmc_execute_ws without a workspace, for a plan that runs as one launch
+ * (bmmc_plan_num_launches is 1): nothing is allocated, and executions of one
+ * plan may overlap.
+ * Errors: INVALID (also for a plan of two launches), ALIAS, ALIGN, CUDA. */
+int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream);
 
 /*
  * End to end with host buffers: copy host_in to dev_in, run the permutation

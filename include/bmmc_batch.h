@@ -2,10 +2,10 @@
  * bmmc_batch.h -- many BMMC permutations in one persistent launch per phase.
  *
  * A batch binds plans[i] (see bmmc.h) to its own input and output arrays.
- * All first passes of the batch (Sec. 5.2: the whole permutation for a
- * one-pass plan, (R L P, 0) for a two-pass plan) run as one launch per
- * element size present; all second passes ((U R, c)) run as a second such
- * launch.  Each launch is a persistent grid of (SMs x resident blocks) thread
+ * All first passes of the batch (the whole permutation for a plan of one
+ * launch, see bmmc_plan_num_launches; (R L P, 0) of Sec. 5.2 for the others)
+ * run as one launch per element size present; the second passes ((U R, c)) of
+ * the others run as a second such launch.  Each launch is a persistent grid of (SMs x resident blocks) thread
  * blocks that take chunks of consecutive tiles of the batch, so many small
  * arrays, which cannot fill the GPU one at a time (Sec. 6, arrays under 2^20
  * elements), share the machine, and a batch of any size costs at most six

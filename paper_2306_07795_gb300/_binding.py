@@ -30,10 +30,10 @@ BMMC_PLAN_TMA_LOAD = 2
 # Every entry point declared in include/bmmc.h (checked by the tests).
 EXPORTED = (
     "bmmc_plan_create", "bmmc_plan_create_ex", "bmmc_plan_destroy",
-    "bmmc_plan_num_passes", "bmmc_plan_matrix", "bmmc_plan_pass_matrix",
+    "bmmc_plan_num_passes", "bmmc_plan_num_launches", "bmmc_plan_matrix", "bmmc_plan_pass_matrix",
     "bmmc_plan_inverse",
     "bmmc_plan_workspace_bytes", "bmmc_execute", "bmmc_execute_ws", "bmmc_execute_host",
-    "bmmc_execute_static_ws", "bmmc_plan_verify", "bmmc_plan_describe",
+    "bmmc_execute_direct", "bmmc_execute_static_ws", "bmmc_plan_verify", "bmmc_plan_describe",
     "bmmc_strerror", "bmmc_plan_compose", "bmmc_parm_matrix", "bmmc_execute_ce",
     "bmmc_plan_lift", "bmmc_sort_schedule", "bmmc_device_wait_timeouts",
     # include/bmmc_sort.h
@@ -120,12 +120,14 @@ def lib():
                                  ctypes.POINTER(bmmc_plan_options)]),
         "bmmc_plan_destroy": (None, [vp]),
         "bmmc_plan_num_passes": (ctypes.c_int, [vp]),
+        "bmmc_plan_num_launches": (ctypes.c_int, [vp]),
         "bmmc_plan_matrix": (ctypes.c_int, [vp, u64p, u64p]),
         "bmmc_plan_pass_matrix": (ctypes.c_int, [vp, ctypes.c_int, u64p, u64p]),
         "bmmc_plan_inverse": (ctypes.c_int, [vp, ctypes.POINTER(vp)]),
         "bmmc_plan_workspace_bytes": (ctypes.c_size_t, [vp]),
         "bmmc_execute": (ctypes.c_int, [vp, vp, vp, vp]),
         "bmmc_execute_ws": (ctypes.c_int, [vp, vp, vp, vp, vp]),
+        "bmmc_execute_direct": (ctypes.c_int, [vp, vp, vp, vp]),
         "bmmc_execute_host": (ctypes.c_int, [vp, vp, vp, vp, vp, vp, vp]),
         "bmmc_execute_static_ws": (ctypes.c_int, [vp, vp, vp, vp]),
         "bmmc_plan_verify": (ctypes.c_int, [vp, ctypes.c_uint64]),
@@ -233,6 +235,10 @@ def bmmc_plan_num_passes(h):
     return lib().bmmc_plan_num_passes(h)
 
 
+def bmmc_plan_num_launches(h):
+    return lib().bmmc_plan_num_launches(h)
+
+
 def bmmc_plan_matrix(h, n):
     rows = (ctypes.c_uint64 * n)()
     c = ctypes.c_uint64()
@@ -265,6 +271,10 @@ def bmmc_execute(h, in_ptr, out_ptr, stream=0):
 def bmmc_execute_ws(h, in_ptr, out_ptr, ws_ptr, stream=0):
     _check(lib().bmmc_execute_ws(h, in_ptr, out_ptr, ws_ptr, stream),
            "bmmc_execute_ws")
+
+
+def bmmc_execute_direct(h, in_ptr, out_ptr, stream=0):
+    _check(lib().bmmc_execute_direct(h, in_ptr, out_ptr, stream), "bmmc_execute_direct")
 
 
 def bmmc_execute_host(h, host_in, host_out, dev_in, dev_out, ws_ptr=None, stream=0):

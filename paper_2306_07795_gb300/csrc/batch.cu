@@ -3,10 +3,9 @@
 //
 // A batch binds plans[i] to (ins[i], outs[i]).  Its work is the list of
 // thread-block items of every pass: phase 1 holds the first pass of every
-// plan (in -> out for one-pass plans, in -> workspace slice for two-pass
-// plans), phase 2 the second pass of the two-pass plans (workspace -> out,
-// Sec. 5.2).  Each phase is one persistent kernel per element size present:
-// a grid of (SMs x resident blocks) thread blocks, each walking a contiguous
+// plan (in -> out for plans of one launch, in -> workspace slice for the
+// others), phase 2 the second pass of the latter (workspace -> out,
+// Sec. 5.2).  Each phase is one persistent kernel per element size present: a grid of (SMs x resident blocks) thread blocks, each walking a contiguous
 // range of items, so that small arrays (the paper notes that arrays under
 // 2^20 elements cannot fill a GPU, Sec. 6) share the machine with large ones
 // instead of each needing its own launch.  A block reloads a pass's tables
@@ -482,7 +481,7 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
     uint32_t ndesc = 0;
     for (int i = 0; i < count; ++i) {
         desc0[i] = ndesc++;
-        if (plans[i]->npass == 2) desc1[i] = ndesc++;
+        if (plans[i]->launches() == 2) desc1[i] = ndesc++;
     }
     // Groups in launch order: phase 1 then phase 2, element sizes 4, 8, 16.
     std::vector<Group> groups;
@@ -497,11 +496,11 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
             uint32_t max_smem = 0;
             for (int i = 0; i < count; ++i) {
                 const bmmc_plan p = plans[i];
-                if (p->e_log != e_log || phase >= p->npass) continue;
-                const PassDesc &d = p->desc[phase];
+                if (p->e_log != e_log || phase >= p->launches()) continue;
+                const PassDesc &d = p->launch_desc(phase);
                 BatchEntry en;
                 memset(&en, 0, sizeof(en));
-                if (p->npass == 1) {
+                if (p->launches() == 1) {
                     en.src = (const uint8_t *)ins[i];
                     en.dst = (uint8_t *)outs[i];
                 } else if (phase == 0) {
@@ -562,8 +561,9 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
     // the counters start at zero (uploaded with the tables)
     std::vector<uint8_t> host(desc_bytes + ent_bytes + groups.size() * kCounterBytes, 0);
     for (int i = 0; i < count; ++i) {
-        memcpy(host.data() + (size_t)desc0[i] * kDescSlot, &plans[i]->desc[0], sizeof(PassDesc));
-        if (plans[i]->npass == 2)
+        memcpy(host.data() + (size_t)desc0[i] * kDescSlot, &plans[i]->launch_desc(0),
+               sizeof(PassDesc));
+        if (plans[i]->launches() == 2)
             memcpy(host.data() + (size_t)desc1[i] * kDescSlot, &plans[i]->desc[1],
                    sizeof(PassDesc));
     }

@@ -45,18 +45,40 @@ bool overlap(const void *a, const void *b, uint64_t bytes)
     return x < y + bytes && y < x + bytes;
 }
 
-// Derive the launch tables of pass i of p.
-int derive_one(bmmc_plan_s *p, int i)
+// Derive the launch tables of (t, c) under the options of p.
+int derive_tables(const bmmc_plan_s *p, const f2::Mat &t, uint64_t c, PassDesc *desc,
+                  PassInfo *info)
 {
-    int rc = derive_pass(p->t[i], p->tc[i], p->n, p->e_log, p->opt, &p->desc[i], &p->info[i]);
-    if (rc == 0 && p->opt.swizzle128 && !p->desc[i].tma) {
+    int rc = derive_pass(t, c, p->n, p->e_log, p->opt, desc, info);
+    if (rc == 0 && p->opt.swizzle128 && !desc->tma) {
         // the fixed swizzle did not give conflict-free gathers: this pass
         // keeps the searched swizzle and 16-byte copies
         PlanOptions o2 = p->opt;
         o2.swizzle128 = false;
-        rc = derive_pass(p->t[i], p->tc[i], p->n, p->e_log, o2, &p->desc[i], &p->info[i]);
+        rc = derive_pass(t, c, p->n, p->e_log, o2, desc, info);
     }
     return rc;
+}
+
+// Derive the launch tables of pass i of p.
+int derive_one(bmmc_plan_s *p, int i)
+{
+    return derive_tables(p, p->t[i], p->tc[i], &p->desc[i], &p->info[i]);
+}
+
+// The tables of every pass, for the queries: a fused plan derives those of
+// its factors here, on first use.
+int need_passes(bmmc_plan_s *p)
+{
+    if (p->derived < p->npass) return BMMC_ERR_INVALID;
+    if (!p->fused) return BMMC_OK;
+    std::lock_guard<std::mutex> lock(p->derive_mu);
+    for (int i = 0; i < p->npass && !p->factors_derived; ++i) {
+        const int rc = derive_one(p, i);
+        if (rc) return rc;
+    }
+    p->factors_derived = true;
+    return BMMC_OK;
 }
 
 // derive_passes: how many passes get their tables now (the rest later, by
@@ -130,7 +152,23 @@ int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
         p->t[1] = t1;  // then (U R, c)
         p->tc[1] = c;
     }
-    for (int i = 0; i < p->npass && i < derive_passes; ++i) {
+    // A two-pass plan whose (A, c) has tables of its own (tiles that are
+    // cosets of Lo + ker A_hi, as BMMC_PLAN_SINGLE_PASS uses) runs as that one
+    // launch: the product of the two passes in half their traffic, the same
+    // bytes.  Measured on GB300, dense A, one launch against two in a graph:
+    // 3.5 / 7.0 us at 1 MiB, 7.8 / 17.9 us at 32 MiB, 40.8 / 79 us at 256 MiB,
+    // 313 / 625 us at 1 GiB and 4.93 / 9.87 ms at 16 GiB; from 128 KiB to
+    // 32 GiB at every element size one launch took 0.43 to 0.53 of two.
+    // With the default segments the factors' tables always exist (a tile has
+    // at most 2^(16 - e_log) bytes), so creation cannot fail for want of
+    // them and only queries derive them.  Chosen segments are the caller's
+    // tiles for the two passes, which then run as asked.
+    if (p->npass == 2 && opt.seg_bits == 0 &&
+        derive_tables(p, a, c, &p->whole, &p->whole_info) == 0) {
+        p->fused = true;
+        p->derived = 2;
+    }
+    for (int i = p->derived; i < p->npass && i < derive_passes; ++i) {
         int rc = derive_one(p, i);
         if (rc) {
             delete p;
@@ -142,22 +180,26 @@ int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
     return BMMC_OK;
 }
 
-// key: comparator epilogue of the last pass (0 = none).
+// key: comparator epilogue of the last pass (0 = none).  need_ws: a two-pass
+// plan is refused without a workspace, also when its one launch would not
+// touch it.
 int execute_impl(bmmc_plan p, const void *in, void *out, void *ws, cudaStream_t s,
-                 int key = 0)
+                 int key = 0, bool need_ws = true)
 {
     const uint64_t bytes = array_bytes(p);
     if (p->derived < p->npass) return BMMC_ERR_INVALID;
     if (((uintptr_t)in | (uintptr_t)out) & 15u) return BMMC_ERR_ALIGN;
     if (overlap(in, out, bytes)) return BMMC_ERR_ALIAS;
-    if (p->npass == 1) {
+    if (p->npass == 2 && need_ws) {
+        if (!ws) return BMMC_ERR_INVALID;
+        if ((uintptr_t)ws & 15u) return BMMC_ERR_ALIGN;
+        if (overlap(ws, in, bytes) || overlap(ws, out, bytes)) return BMMC_ERR_ALIAS;
+    }
+    if (p->launches() == 1) {
         if (debug_fail_launch()) return BMMC_ERR_CUDA;
-        cudaError_t err = launch_pass(p->desc[0], in, out, s, key);
+        cudaError_t err = launch_pass(p->launch_desc(0), in, out, s, key);
         return err == cudaSuccess ? BMMC_OK : BMMC_ERR_CUDA;
     }
-    if (!ws) return BMMC_ERR_INVALID;
-    if ((uintptr_t)ws & 15u) return BMMC_ERR_ALIGN;
-    if (overlap(ws, in, bytes) || overlap(ws, out, bytes)) return BMMC_ERR_ALIAS;
     if (debug_fail_launch()) return BMMC_ERR_CUDA;
     cudaError_t err = launch_pass(p->desc[0], in, ws, s, 0);
     if (err != cudaSuccess) return BMMC_ERR_CUDA;
@@ -232,6 +274,8 @@ void bmmc_plan_destroy(bmmc_plan p)
 }
 
 int bmmc_plan_num_passes(bmmc_plan p) { return p ? p->npass : BMMC_ERR_INVALID; }
+
+int bmmc_plan_num_launches(bmmc_plan p) { return p ? p->launches() : BMMC_ERR_INVALID; }
 
 int bmmc_plan_matrix(bmmc_plan p, uint64_t *rows_out, uint64_t *c_out)
 {
@@ -355,6 +399,12 @@ int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws, bmmc_strea
     return execute_impl(p, in, out, ws, (cudaStream_t)stream);
 }
 
+int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream)
+{
+    if (!p || !in || !out || p->launches() != 1) return BMMC_ERR_INVALID;
+    return execute_impl(p, in, out, nullptr, (cudaStream_t)stream, 0, false);
+}
+
 int bmmc_execute_host(bmmc_plan p, const void *host_in, void *host_out, void *dev_in,
                       void *dev_out, void *ws, bmmc_stream_t stream)
 {
@@ -413,7 +463,16 @@ namespace {
 
 int verify_impl(bmmc_plan p, uint64_t max_ctas)
 {
-    if (!p || p->derived < p->npass) return BMMC_ERR_INVALID;
+    if (!p) return BMMC_ERR_INVALID;
+    const int rc = need_passes(p);
+    if (rc) return rc;
+    if (p->fused) {
+        std::string why;
+        if (verify_pass(p->whole, p->a, p->c, max_ctas, &why) != 0) {
+            fprintf(stderr, "bmmc_plan_verify: fused pass: %s\n", why.c_str());
+            return BMMC_ERR_UNSUPPORTED;
+        }
+    }
     for (int i = 0; i < p->npass; ++i) {
         std::string why;
         if (verify_pass(p->desc[i], p->t[i], p->tc[i], max_ctas, &why) != 0) {
@@ -436,33 +495,38 @@ int verify_impl(bmmc_plan p, uint64_t max_ctas)
     return BMMC_OK;
 }
 
+std::string pass_json(const PassDesc &d, const PassInfo &f)
+{
+    char tmp[512];
+    snprintf(tmp, sizeof(tmp),
+             "{\"naive\": %u, \"tiled\": %d, \"seg_bits\": %u, \"row_bits\": %u, "
+             "\"n_over\": %d, \"tiles_per_block_log2\": %u, \"blocks\": %llu, "
+             "\"threads\": %u, \"loop\": %u, \"smem_bytes\": %u, "
+             "\"wavefronts_load\": %d, \"ideal_load\": %d, \"wavefronts_store\": %d, "
+             "\"ideal_store\": %d, \"lanes34\": [%d, %d], \"rot\": %d, "
+             "\"sigma\": [%u, %u, %u], \"tma\": %u}",
+             d.naive, f.tiled, d.k, d.m, f.n_over, d.it, (unsigned long long)(1ull << d.n_cta),
+             1u << d.thread_bits, d.loop, d.smem_bytes, f.wavefronts_load, f.ideal_load,
+             f.wavefronts_store, f.ideal_store, f.lane3, f.lane4, f.rot, f.sigma[0], f.sigma[1],
+             f.sigma[2], d.tma);
+    return tmp;
+}
+
 int describe_impl(bmmc_plan p, char *buf, size_t len)
 {
-    if (!p || p->derived < p->npass) return BMMC_ERR_INVALID;
+    if (!p) return BMMC_ERR_INVALID;
+    const int rc = need_passes(p);
+    if (rc) return rc;
     std::string s = "{\"n\": " + std::to_string(p->n) +
                     ", \"elem_bytes\": " + std::to_string(1 << p->e_log) +
                     ", \"strategy\": \"" +
                     ((p->opt.flags & BMMC_PLAN_SINGLE_PASS) ? "single_pass" : "paper") +
-                    "\", \"passes\": [";
-    for (int i = 0; i < p->npass; ++i) {
-        const PassDesc &d = p->desc[i];
-        const PassInfo &f = p->info[i];
-        char tmp[512];
-        snprintf(tmp, sizeof(tmp),
-                 "%s{\"naive\": %u, \"tiled\": %d, \"seg_bits\": %u, \"row_bits\": %u, "
-                 "\"n_over\": %d, \"tiles_per_block_log2\": %u, \"blocks\": %llu, "
-                 "\"threads\": %u, \"loop\": %u, \"smem_bytes\": %u, "
-                 "\"wavefronts_load\": %d, \"ideal_load\": %d, \"wavefronts_store\": %d, "
-                 "\"ideal_store\": %d, \"lanes34\": [%d, %d], \"rot\": %d, "
-                 "\"sigma\": [%u, %u, %u], \"tma\": %u}",
-                 i ? ", " : "", d.naive, f.tiled, d.k, d.m, f.n_over, d.it,
-                 (unsigned long long)(1ull << d.n_cta), 1u << d.thread_bits, d.loop,
-                 d.smem_bytes, f.wavefronts_load, f.ideal_load, f.wavefronts_store,
-                 f.ideal_store, f.lane3, f.lane4, f.rot, f.sigma[0], f.sigma[1],
-                 f.sigma[2], d.tma);
-        s += tmp;
-    }
-    s += "]}";
+                    "\", \"launches\": " + std::to_string(p->launches()) + ", \"passes\": [";
+    for (int i = 0; i < p->npass; ++i)
+        s += (i ? ", " : "") + pass_json(p->desc[i], p->info[i]);
+    s += "]";
+    if (p->fused) s += ", \"fused\": " + pass_json(p->whole, p->whole_info);
+    s += "}";
     if (buf && len) {
         size_t cpy = s.size() < len - 1 ? s.size() : len - 1;
         memcpy(buf, s.data(), cpy);

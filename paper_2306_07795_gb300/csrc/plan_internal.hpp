@@ -26,12 +26,24 @@ struct bmmc_plan_s {
     // API has all of them; the request server derives the second pass of a
     // two-pass plan after launching the first (plan_create_first_pass).
     int derived = 0;
+    // A two-pass plan whose permutation runs as one launch: `whole` holds the
+    // tables of (A, c) over generic tiles (see create_impl in capi.cpp).  The
+    // two factors' tables then serve the queries only and are derived by the
+    // first one that asks (factors_derived, under derive_mu).
+    bool fused = false;
+    bmmc::PassDesc whole;
+    bmmc::PassInfo whole_info;
+    std::mutex derive_mu;
+    bool factors_derived = false;
     // Workspace owned by the plan for bmmc_execute (two-pass plans only).
     std::mutex ws_mu;
     void *ws = nullptr;
     int ws_device = -1;
 
     uint64_t bytes() const { return (1ull << n) << e_log; }
+    // Kernel launches of one execution, and the tables of launch i.
+    int launches() const { return fused ? 1 : npass; }
+    const bmmc::PassDesc &launch_desc(int i) const { return fused ? whole : desc[i]; }
 };
 
 namespace bmmc {

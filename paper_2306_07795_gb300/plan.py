@@ -22,7 +22,7 @@ class Plan:
 
     rows: n row masks (bit j of rows[i] is a_ij); c: complement mask.
     flags: BMMC_PLAN_PAPER (one tiled pass, or two after the UL.P
-    factorisation) or BMMC_PLAN_SINGLE_PASS.
+    factorisation, run fused as one launch) or BMMC_PLAN_SINGLE_PASS.
     """
 
     def __init__(self, n, rows, c=0, elem_bytes=4, flags=B.BMMC_PLAN_PAPER,
@@ -43,6 +43,7 @@ class Plan:
                                             cta_tile_log2, tile_order)
         self._inverse = None
         self._ws_bytes = None
+        self._direct = B.bmmc_plan_num_launches(self._h) == 1
 
     # -- plan queries -------------------------------------------------------
     @property
@@ -56,6 +57,11 @@ class Plan:
     @property
     def num_passes(self):
         return B.bmmc_plan_num_passes(self._h)
+
+    @property
+    def num_launches(self):
+        """Kernel launches one execution makes (1 when two passes run fused)."""
+        return B.bmmc_plan_num_launches(self._h)
 
     @property
     def workspace_bytes(self):
@@ -113,18 +119,25 @@ class Plan:
             self._check_tensor(out, "out")
         dev = x.device
         raw = stream.cuda_stream if stream is not None else _current_raw_stream(dev)
-        ws_bytes = self._ws_bytes
-        if ws_bytes is None:
-            ws_bytes = self._ws_bytes = self.workspace_bytes  # plans are immutable
-        if ws_bytes and workspace is None:
-            workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
-        ws_ptr = workspace.data_ptr() if ws_bytes else None
+        if workspace is None and self._direct:
+            def run():
+                return B.lib().bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), raw)
+        else:
+            ws_bytes = self._ws_bytes
+            if ws_bytes is None:
+                ws_bytes = self._ws_bytes = self.workspace_bytes  # plans are immutable
+            if ws_bytes and workspace is None:
+                workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
+            ws_ptr = workspace.data_ptr() if ws_bytes else None
+
+            def run():
+                return B.lib().bmmc_execute_ws(self._h, x.data_ptr(), out.data_ptr(), ws_ptr,
+                                               raw)
         if dev.index == torch.cuda.current_device():
-            code = B.lib().bmmc_execute_ws(self._h, x.data_ptr(), out.data_ptr(), ws_ptr, raw)
+            code = run()
         else:
             with torch.cuda.device(dev):
-                code = B.lib().bmmc_execute_ws(self._h, x.data_ptr(), out.data_ptr(),
-                                               ws_ptr, raw)
+                code = run()
         if code != B.BMMC_OK:
             raise B.BmmcError(code, "bmmc_execute_ws")
         return out

@@ -1,0 +1,61 @@
+"""Two-pass plans that run as one launch: which plans do, and that the launch
+moves every element as the two passes do."""
+
+import pytest
+
+import oracle
+from oracle import f2
+import paper_2306_07795_gb300 as bm
+import workloads as wl
+
+
+def _inv(rows):
+    return f2.is_invertible(rows, len(rows))
+
+
+def _dense(n, seed):
+    return wl.dense_bmmc(n, seed, _inv)
+
+
+@pytest.mark.parametrize("e,n", [(4, 15), (4, 20), (8, 14), (8, 19), (16, 13), (16, 18)])
+def test_rule(e, n):
+    """Default segments: one launch, whose tables are walked with the passes';
+    chosen segments: the two passes as asked; both keep the two matrices."""
+    rows, c = _dense(n, n + e)
+    for kw in ({}, {"cta_tile_log2": 12}, {"cta_tile_log2": 16, "tile_order": 2},
+               {"flags": bm.BMMC_PLAN_TMA_LOAD}):
+        p = bm.Plan(n, rows, c, e, **kw)
+        assert (p.num_passes, p.num_launches) == (2, 1)
+        assert p.workspace_bytes == p.nbytes
+        assert p.verify() == 0
+        d = p.describe()
+        assert d["launches"] == 1 and len(d["passes"]) == 2 and "fused" in d
+    q = bm.Plan(n, rows, c, e, seg_bits=8 - (e.bit_length() - 1))
+    assert (q.num_passes, q.num_launches) == (2, 2)
+    assert q.pass_matrices() == p.pass_matrices()
+    assert q.verify() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("e,n", [(4, 15), (4, 22), (8, 14), (8, 20), (16, 13), (16, 19)])
+def test_direct_equals_workspace_form(e, n):
+    import torch
+    rows, c = _dense(n, 3 * n + e)
+    x = wl.payload_torch(n, e, seed=n)
+    p = bm.Plan(n, rows, c, e)
+    q = bm.Plan(n, rows, c, e, seg_bits=8 - (e.bit_length() - 1))  # two launches
+    a, b = torch.full_like(x, -1), torch.full_like(x, -1)
+    s = torch.cuda.current_stream().cuda_stream
+    bm.bmmc_execute_direct(p.handle, x.data_ptr(), a.data_ptr(), s)
+    q(x, out=b)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
+    assert oracle.count_mismatch(n, rows, c, x.cpu().numpy(), a.cpu().numpy(), elem_bytes=e) == 0
+    for h, i, o, code in ((q.handle, x, a, bm.BMMC_ERR_INVALID),
+                          (p.handle, x, x, bm.BMMC_ERR_ALIAS)):
+        with pytest.raises(bm.BmmcError) as ei:
+            bm.bmmc_execute_direct(h, i.data_ptr(), o.data_ptr(), s)
+        assert ei.value.code == code
+    with pytest.raises(bm.BmmcError) as ei:
+        bm.bmmc_execute_ws(p.handle, x.data_ptr(), a.data_ptr(), None, s)
+    assert ei.value.code == bm.BMMC_ERR_INVALID  # a workspace is still asked for here
