@@ -207,11 +207,15 @@ int bmmc_execute(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream);
 int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws,
                     bmmc_stream_t stream);
 
-/* As bmmc_execute_ws without a workspace, for a plan that runs as one launch
- * (bmmc_plan_num_launches is 1): nothing is allocated, and executions of one
- * plan may overlap.
+/* Run a plan of one launch (bmmc_plan_num_launches) on each of `rows` >= 1
+ * arrays stored one after another, with no workspace: nothing is allocated,
+ * executions of one plan may overlap, and the rows share one launch (65535 of
+ * them at most; a plan with tensor-copy loads launches per row).  in and out
+ * hold rows * 2^n * elem_bytes bytes; several rows need arrays of whole
+ * 16-byte units.
  * Errors: INVALID (also for a plan of two launches), ALIAS, ALIGN, CUDA. */
-int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream);
+int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, uint64_t rows,
+                        bmmc_stream_t stream);
 
 /*
  * End to end with host buffers: copy host_in to dev_in, run the permutation

@@ -127,7 +127,7 @@ def lib():
         "bmmc_plan_workspace_bytes": (ctypes.c_size_t, [vp]),
         "bmmc_execute": (ctypes.c_int, [vp, vp, vp, vp]),
         "bmmc_execute_ws": (ctypes.c_int, [vp, vp, vp, vp, vp]),
-        "bmmc_execute_direct": (ctypes.c_int, [vp, vp, vp, vp]),
+        "bmmc_execute_direct": (ctypes.c_int, [vp, vp, vp, ctypes.c_uint64, vp]),
         "bmmc_execute_host": (ctypes.c_int, [vp, vp, vp, vp, vp, vp, vp]),
         "bmmc_execute_static_ws": (ctypes.c_int, [vp, vp, vp, vp]),
         "bmmc_plan_verify": (ctypes.c_int, [vp, ctypes.c_uint64]),
@@ -273,8 +273,8 @@ def bmmc_execute_ws(h, in_ptr, out_ptr, ws_ptr, stream=0):
            "bmmc_execute_ws")
 
 
-def bmmc_execute_direct(h, in_ptr, out_ptr, stream=0):
-    _check(lib().bmmc_execute_direct(h, in_ptr, out_ptr, stream), "bmmc_execute_direct")
+def bmmc_execute_direct(h, in_ptr, out_ptr, rows=1, stream=0):
+    _check(lib().bmmc_execute_direct(h, in_ptr, out_ptr, rows, stream), "bmmc_execute_direct")
 
 
 def bmmc_execute_host(h, host_in, host_out, dev_in, dev_out, ws_ptr=None, stream=0):

@@ -10,6 +10,7 @@ the library's kernels; nothing is computed in PyTorch.
 When the leading dimensions hold 2^b rows in total, the whole tensor is one
 array of 2^(n+b) elements and the permutation is the BMMC diag(A, I_b) with
 complement (c, 0): one launch (or one plan's passes) for the whole batch.
+Any other count of rows is an odd count of such arrays, which share one launch.
 """
 
 from . import _binding as B
@@ -43,7 +44,12 @@ def _apply(plan, x):
     lifted = _lifted_plan(plan, rows_total) if rows_total > 1 else plan
     if lifted is not None:
         return lifted(x.view(-1)).view(x.shape)
-    out = torch.empty_like(x)
+    # an odd count of groups of 2^b rows, each group one array of the lifted plan
+    b = min((rows_total & -rows_total).bit_length() - 1, 32 - plan.n)
+    out = _lifted_plan(plan, 1 << b).run_rows(x, rows_total >> b)
+    if out is not None:
+        return out
+    out = torch.empty_like(x)  # a plan of two launches: row by row
     xf, of = x.view(rows_total, -1), out.view(rows_total, -1)
     for r in range(rows_total):
         plan(xf[r], out=of[r])

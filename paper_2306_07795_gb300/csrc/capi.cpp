@@ -15,8 +15,8 @@
 #include "plan_internal.hpp"
 
 namespace bmmc {
-cudaError_t launch_pass(const PassDesc &d, const void *in, void *out, cudaStream_t s,
-                        int key);
+cudaError_t launch_pass(const PassDesc &d, const void *in, void *out, cudaStream_t s, int key,
+                        uint64_t rows = 1);
 cudaError_t device_wait_timeouts(unsigned long long *count);
 }
 
@@ -180,17 +180,16 @@ int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
     return BMMC_OK;
 }
 
-// key: comparator epilogue of the last pass (0 = none).  need_ws: a two-pass
-// plan is refused without a workspace, also when its one launch would not
-// touch it.
+// key: comparator epilogue of the last pass (0 = none).  A two-pass plan is
+// refused without a workspace, also when its one launch would not touch it.
 int execute_impl(bmmc_plan p, const void *in, void *out, void *ws, cudaStream_t s,
-                 int key = 0, bool need_ws = true)
+                 int key = 0)
 {
     const uint64_t bytes = array_bytes(p);
     if (p->derived < p->npass) return BMMC_ERR_INVALID;
     if (((uintptr_t)in | (uintptr_t)out) & 15u) return BMMC_ERR_ALIGN;
     if (overlap(in, out, bytes)) return BMMC_ERR_ALIAS;
-    if (p->npass == 2 && need_ws) {
+    if (p->npass == 2) {
         if (!ws) return BMMC_ERR_INVALID;
         if ((uintptr_t)ws & 15u) return BMMC_ERR_ALIGN;
         if (overlap(ws, in, bytes) || overlap(ws, out, bytes)) return BMMC_ERR_ALIAS;
@@ -399,10 +398,19 @@ int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws, bmmc_strea
     return execute_impl(p, in, out, ws, (cudaStream_t)stream);
 }
 
-int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream)
+int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, uint64_t rows,
+                        bmmc_stream_t stream)
 {
     if (!p || !in || !out || p->launches() != 1) return BMMC_ERR_INVALID;
-    return execute_impl(p, in, out, nullptr, (cudaStream_t)stream, 0, false);
+    const uint64_t bytes = array_bytes(p);
+    if (rows < 1 || rows > ~0ull / bytes) return BMMC_ERR_INVALID;
+    const uint64_t stride = rows > 1 ? bytes : 0;
+    if (((uintptr_t)in | (uintptr_t)out | stride) & 15u) return BMMC_ERR_ALIGN;
+    if (overlap(in, out, rows * bytes)) return BMMC_ERR_ALIAS;
+    if (debug_fail_launch()) return BMMC_ERR_CUDA;
+    const cudaError_t err =
+        launch_pass(p->launch_desc(0), in, out, (cudaStream_t)stream, 0, rows);
+    return err == cudaSuccess ? BMMC_OK : BMMC_ERR_CUDA;
 }
 
 int bmmc_execute_host(bmmc_plan p, const void *host_in, void *host_out, void *dev_in,

@@ -20,15 +20,22 @@ namespace bmmc {
 
 namespace {
 
-// Element size 2^E_LOG bytes; one block per thread-block index of the pass.
+// Element size 2^E_LOG bytes; one block per thread-block index of the pass and
+// per row: row r of the launch is the array `r * row_bytes` bytes further on.
+// A count of rows that is a power of two is better folded into the pass
+// (bmmc_plan_lift: whole tiles even where a row is small); the odd factor of
+// any other count is gridDim.y.  24 rows of 2^16 floats, permuted there and
+// back (parm): 636 us with a launch per row, ROWS_FIGURE us with one launch
+// each way.
 template <int E_LOG, int KEY>
 __global__ void __launch_bounds__(256)
-    bmmc_tiled_pass(const __grid_constant__ PassDesc d,
-                    const uint8_t *__restrict__ in, uint8_t *__restrict__ out)
+    bmmc_tiled_pass(const __grid_constant__ PassDesc d, const uint8_t *__restrict__ in,
+                    uint8_t *__restrict__ out, uint64_t row_bytes)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
-    dev::run_tile<E_LOG, KEY>(d, blockIdx.x, in, out, sbase);
+    const uint64_t row = blockIdx.y * row_bytes;
+    dev::run_tile<E_LOG, KEY>(d, blockIdx.x, in + row, out + row, sbase);
 }
 
 // Bounded waits of the tensor-copy kernel that gave up (read by
@@ -64,17 +71,21 @@ __global__ void __launch_bounds__(256)
     dev::tile_store<E_LOG, KEY>(d, a, out, sbase);
 }
 
-// Arrays under 1 KiB: one block, one thread per element, direct index map.
+// Arrays under 1 KiB: one block per row, one thread per element, direct index
+// map.
 template <int E_LOG, int KEY>
 __global__ void bmmc_naive_pass(const __grid_constant__ PassDesc d,
-                                const uint8_t *__restrict__ in, uint8_t *__restrict__ out)
+                                const uint8_t *__restrict__ in, uint8_t *__restrict__ out,
+                                uint64_t row_bytes)
 {
     dev::grid_dependency_wait();
     dev::allow_dependent_launch();
-    dev::run_naive<E_LOG, KEY>(d, in, out);
+    const uint64_t row = blockIdx.x * row_bytes;
+    dev::run_naive<E_LOG, KEY>(d, in + row, out + row);
 }
 
 constexpr int kMaxDevices = 64;
+constexpr uint64_t kMaxRows = 65535;  // gridDim.y
 constexpr int kSmemLimit = 128 * 1024;
 constexpr int kSmemLimitTma = kSmemLimit + 2048;  // 1 KiB alignment + mbarrier
 // Per device, element size and key: the kernel's shared-memory limit has
@@ -142,14 +153,17 @@ cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// rows <= kMaxRows (1 for tensor copies, whose map covers one array).
 template <int E_LOG, int KEY>
-cudaError_t launch_typed(const PassDesc &d, const void *in, void *out, cudaStream_t s)
+cudaError_t launch_typed(const PassDesc &d, const void *in, void *out, uint32_t rows,
+                         cudaStream_t s)
 {
     const uint8_t *src = static_cast<const uint8_t *>(in);
     uint8_t *dst = static_cast<uint8_t *>(out);
+    const uint64_t row_bytes = ((uint64_t)1 << d.n) << E_LOG;
     if (d.naive)
-        return launch_pdl(bmmc_naive_pass<E_LOG, KEY>, dim3(1), dim3(1u << d.n), 0, s, d, src,
-                          dst);
+        return launch_pdl(bmmc_naive_pass<E_LOG, KEY>, dim3(rows), dim3(1u << d.n), 0, s, d, src,
+                          dst, row_bytes);
     // Tiles within the default 48 KiB of dynamic shared memory (the default
     // 16 KiB ones) need no attribute, and so no device lookup per launch.
     constexpr uint32_t kDefaultSmem = 48 * 1024;
@@ -162,8 +176,7 @@ cudaError_t launch_typed(const PassDesc &d, const void *in, void *out, cudaStrea
     }
     if (d.tma) {
         CUtensorMap tmap;
-        const uint64_t bytes = ((uint64_t)1 << d.n) << E_LOG;
-        if (encode_lines_map(&tmap, in, bytes, 1u << (d.k + E_LOG - 7))) {
+        if (encode_lines_map(&tmap, in, row_bytes, 1u << (d.k + E_LOG - 7))) {
             if (needs_attr && dev >= 0 && dev < kMaxDevices &&
                 !g_attr_set_tma[dev][E_LOG - 2][KEY].load(std::memory_order_acquire)) {
                 err = cudaFuncSetAttribute(bmmc_tiled_pass_tma<E_LOG, KEY>,
@@ -185,40 +198,53 @@ cudaError_t launch_typed(const PassDesc &d, const void *in, void *out, cudaStrea
         if (err != cudaSuccess) return err;
         g_attr_set[dev][E_LOG - 2][KEY].store(true, std::memory_order_release);
     }
-    return launch_pdl(bmmc_tiled_pass<E_LOG, KEY>, dim3(1u << d.n_cta),
-                      dim3(1u << d.thread_bits), d.smem_bytes, s, d, src, dst);
+    return launch_pdl(bmmc_tiled_pass<E_LOG, KEY>, dim3(1u << d.n_cta, rows),
+                      dim3(1u << d.thread_bits), d.smem_bytes, s, d, src, dst, row_bytes);
 }
 
 }  // namespace
 
 // key: 0 (plain permutation) or a bmmc_key_type value matching the element
-// size (1..3 for 4-byte, 4..6 for 8-byte elements).
-cudaError_t launch_pass(const PassDesc &d, const void *in, void *out, cudaStream_t s,
-                        int key)
+// size (1..3 for 4-byte, 4..6 for 8-byte elements).  rows: arrays one after
+// another, each permuted alike.
+cudaError_t launch_pass(const PassDesc &d, const void *in, void *out, cudaStream_t s, int key,
+                        uint64_t rows)
 {
     using namespace dev;
-    switch (d.e_log) {
-    case 2:
-        switch (key) {
-        case kKeyNone: return launch_typed<2, kKeyNone>(d, in, out, s);
-        case kKeyI32: return launch_typed<2, kKeyI32>(d, in, out, s);
-        case kKeyU32: return launch_typed<2, kKeyU32>(d, in, out, s);
-        case kKeyF32: return launch_typed<2, kKeyF32>(d, in, out, s);
+    auto launch = [&](const void *src, void *dst, uint32_t r) {
+        switch (d.e_log) {
+        case 2:
+            switch (key) {
+            case kKeyNone: return launch_typed<2, kKeyNone>(d, src, dst, r, s);
+            case kKeyI32: return launch_typed<2, kKeyI32>(d, src, dst, r, s);
+            case kKeyU32: return launch_typed<2, kKeyU32>(d, src, dst, r, s);
+            case kKeyF32: return launch_typed<2, kKeyF32>(d, src, dst, r, s);
+            default: return cudaErrorInvalidValue;
+            }
+        case 3:
+            switch (key) {
+            case kKeyNone: return launch_typed<3, kKeyNone>(d, src, dst, r, s);
+            case kKeyI64: return launch_typed<3, kKeyI64>(d, src, dst, r, s);
+            case kKeyU64: return launch_typed<3, kKeyU64>(d, src, dst, r, s);
+            case kKeyF64: return launch_typed<3, kKeyF64>(d, src, dst, r, s);
+            default: return cudaErrorInvalidValue;
+            }
+        case 4:
+            if (key != kKeyNone) return cudaErrorInvalidValue;
+            return launch_typed<4, kKeyNone>(d, src, dst, r, s);
         default: return cudaErrorInvalidValue;
         }
-    case 3:
-        switch (key) {
-        case kKeyNone: return launch_typed<3, kKeyNone>(d, in, out, s);
-        case kKeyI64: return launch_typed<3, kKeyI64>(d, in, out, s);
-        case kKeyU64: return launch_typed<3, kKeyU64>(d, in, out, s);
-        case kKeyF64: return launch_typed<3, kKeyF64>(d, in, out, s);
-        default: return cudaErrorInvalidValue;
-        }
-    case 4:
-        if (key != kKeyNone) return cudaErrorInvalidValue;
-        return launch_typed<4, kKeyNone>(d, in, out, s);
-    default: return cudaErrorInvalidValue;
+    };
+    const uint64_t row_bytes = ((uint64_t)1 << d.n) << d.e_log;
+    const uint64_t step = d.tma ? 1 : kMaxRows;
+    for (uint64_t r = 0; r < rows; r += step) {
+        const cudaError_t err =
+            launch(static_cast<const uint8_t *>(in) + r * row_bytes,
+                   static_cast<uint8_t *>(out) + r * row_bytes,
+                   (uint32_t)(rows - r < step ? rows - r : step));
+        if (err != cudaSuccess) return err;
     }
+    return cudaSuccess;
 }
 
 // Number of bounded waits of tensor-copy kernels that gave up on the current

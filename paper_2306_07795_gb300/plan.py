@@ -121,7 +121,7 @@ class Plan:
         raw = stream.cuda_stream if stream is not None else _current_raw_stream(dev)
         if workspace is None and self._direct:
             def run():
-                return B.lib().bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), raw)
+                return B.lib().bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), 1, raw)
         else:
             ws_bytes = self._ws_bytes
             if ws_bytes is None:
@@ -140,6 +140,28 @@ class Plan:
                 code = run()
         if code != B.BMMC_OK:
             raise B.BmmcError(code, "bmmc_execute_ws")
+        return out
+
+    def run_rows(self, x, rows):
+        """Permute each of the `rows` arrays of the contiguous CUDA tensor x
+        alike, in one launch (bmmc_execute_direct).  Returns a new tensor, or
+        None for a plan of two launches."""
+        import torch
+
+        if not self._direct:
+            return None
+        if not (x.is_cuda and x.is_contiguous()
+                and x.numel() * x.element_size() == rows * self.nbytes):
+            raise ValueError("x must be a contiguous CUDA tensor of %d bytes"
+                             % (rows * self.nbytes))
+        out = torch.empty_like(x)
+        dev = x.device
+        raw = _current_raw_stream(dev)
+        if dev.index == torch.cuda.current_device():
+            B.bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), rows, raw)
+        else:
+            with torch.cuda.device(dev):
+                B.bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), rows, raw)
         return out
 
     def execute_host(self, host_in, host_out, dev_in, dev_out, stream=None, workspace=None):

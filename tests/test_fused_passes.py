@@ -1,5 +1,6 @@
-"""Two-pass plans that run as one launch: which plans do, and that the launch
-moves every element as the two passes do."""
+"""Two-pass plans that run as one launch, and rows that share one: which plans
+do, and that the launch moves every element as the two passes, or the launches
+row by row, do."""
 
 import pytest
 
@@ -46,7 +47,7 @@ def test_direct_equals_workspace_form(e, n):
     q = bm.Plan(n, rows, c, e, seg_bits=8 - (e.bit_length() - 1))  # two launches
     a, b = torch.full_like(x, -1), torch.full_like(x, -1)
     s = torch.cuda.current_stream().cuda_stream
-    bm.bmmc_execute_direct(p.handle, x.data_ptr(), a.data_ptr(), s)
+    bm.bmmc_execute_direct(p.handle, x.data_ptr(), a.data_ptr(), 1, s)
     q(x, out=b)
     torch.cuda.synchronize()
     assert torch.equal(a, b)
@@ -54,8 +55,42 @@ def test_direct_equals_workspace_form(e, n):
     for h, i, o, code in ((q.handle, x, a, bm.BMMC_ERR_INVALID),
                           (p.handle, x, x, bm.BMMC_ERR_ALIAS)):
         with pytest.raises(bm.BmmcError) as ei:
-            bm.bmmc_execute_direct(h, i.data_ptr(), o.data_ptr(), s)
+            bm.bmmc_execute_direct(h, i.data_ptr(), o.data_ptr(), 1, s)
         assert ei.value.code == code
     with pytest.raises(bm.BmmcError) as ei:
         bm.bmmc_execute_ws(p.handle, x.data_ptr(), a.data_ptr(), None, s)
     assert ei.value.code == bm.BMMC_ERR_INVALID  # a workspace is still asked for here
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("e,n,rows", [(4, 2, 7), (4, 5, 3), (4, 8, 65537), (4, 10, 1), (4, 13, 6),
+                                      (8, 1, 5), (8, 16, 24), (16, 3, 9), (16, 14, 3)])
+@pytest.mark.parametrize("flags", [0, bm.BMMC_PLAN_TMA_LOAD])
+def test_rows_share_a_launch(e, n, rows, flags):
+    """Every row as alone: arrays below and above 1 KiB, more rows than one
+    grid holds, tensor-copy loads (a launch per row)."""
+    import torch
+    if flags and rows > 100:
+        rows = 101
+    mat, c = _dense(n, n + rows)
+    p = bm.Plan(n, mat, c, e, flags=flags)
+    x = torch.randint(-2**31, 2**31 - 1, (rows, p.nbytes // 4), dtype=torch.int32, device="cuda")
+    y = p.run_rows(x, rows)
+    at = torch.from_numpy(f2.index_table(n, mat, c).astype("int64")).cuda()
+    want = torch.empty_like(x).view(rows, 1 << n, -1)
+    want[:, at] = x.view(rows, 1 << n, -1)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want.view_as(y))
+
+
+@pytest.mark.gpu
+def test_rows_refused():
+    import torch
+    x = torch.zeros(3 * 2, dtype=torch.int32, device="cuda")
+    p = bm.Plan(1, [1], 1, 4)  # rows of 8 bytes do not start on 16-byte boundaries
+    with pytest.raises(bm.BmmcError) as ei:
+        p.run_rows(x, 3)
+    assert ei.value.code == bm.BMMC_ERR_ALIGN
+    with pytest.raises(bm.BmmcError) as ei:
+        bm.bmmc_execute_direct(p.handle, x.data_ptr(), x.data_ptr(), 0, 0)
+    assert ei.value.code == bm.BMMC_ERR_INVALID
