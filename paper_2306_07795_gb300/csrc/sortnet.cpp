@@ -20,7 +20,9 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "bmmc.h"
@@ -168,8 +170,9 @@ extern "C" int bmmc_sort_schedule(int n, uint64_t *stage_rows, int max_stages,
 //   * L_p^{-1} Lo (whole output segments),
 // of dimension at most D (a block holds 2^D keys).  L_0 = I and the last
 // layout is Q_final.  The planner fills each pass with as many consecutive
-// stages as fit, and chooses L_p^{-1} Lo among the partner vectors of the
-// next stages, so that the next pass's input segments cost it no dimension.
+// stages as fit, and chooses L_p^{-1} Lo in the span of the next pass's
+// partner vectors, and in its own where it can, so that the segments cost
+// neither pass a dimension.
 
 namespace bmmc {
 namespace sortnet {
@@ -253,87 +256,199 @@ struct PassPlan {
     std::vector<uint64_t> out;   // basis of L_p^{-1} Lo
 };
 
-// Cut the stages into passes (see above).
-int group_stages(const std::vector<uint64_t> &U, int N, int k, int D,
-                 const std::vector<uint64_t> &o_final, std::vector<PassPlan> *passes)
-{
-    const int S = (int)U.size();
-    std::vector<uint64_t> I;
-    for (int j = 0; j < k; ++j) I.push_back(1ull << j);
-    int s = 0;
-    while (s < S) {
-        PassPlan pp;
-        pp.first = s;
-        std::vector<uint64_t> span = I;
-        int e = s;
-        while (e < S && e - s < kSortMaxStages) {
-            std::vector<uint64_t> t = span;
-            t.push_back(U[e]);
-            if (rank_of(t) > D) break;
-            span.push_back(U[e]);
-            ++e;
+// A subspace of F2^32 as a basis with distinct leading bits.
+struct Span {
+    uint32_t lead[32] = {};  // the basis vector whose leading bit is i, or 0
+    int dim = 0;
+
+    uint32_t reduce(uint32_t v) const
+    {
+        while (v) {
+            const uint32_t b = lead[31 - __builtin_clz(v)];
+            if (!b) break;
+            v ^= b;
         }
-        if (e == S) {
-            // the last pass also writes the final layout's segments
-            auto fits = [&](int end) {
-                std::vector<uint64_t> t = I;
-                for (int q = s; q < end; ++q) t.push_back(U[q]);
-                for (uint64_t v : o_final) t.push_back(v);
-                return rank_of(t) <= D;
-            };
-            const int e_all = e;
-            while (e > s && !fits(e)) --e;
-            if (e == s) e = e_all - 1;  // leave the tail to one more pass
-            if (e == S) {
-                pp.out = o_final;
-                span = I;
-                for (int q = s; q < e; ++q) span.push_back(U[q]);
-                for (uint64_t v : o_final) span.push_back(v);
-            } else {
-                span = I;
-                for (int q = s; q < e; ++q) span.push_back(U[q]);
-            }
-        }
-        if (e == s) return -3;  // D too small to make progress
-        if (pp.out.empty()) {
-            // next pass's input segments: the next stages' partner vectors that
-            // still fit, then vectors of this span
-            std::vector<uint64_t> out;
-            for (int t = e; t < S && t < e + 4 * D && (int)out.size() < k; ++t) {
-                if (in_span(out, U[t])) continue;
-                std::vector<uint64_t> tt = span;
-                tt.insert(tt.end(), out.begin(), out.end());
-                tt.push_back(U[t]);
-                if (rank_of(tt) <= D) out.push_back(U[t]);
-            }
-            for (size_t q = 0; q < span.size() && (int)out.size() < k; ++q)
-                if (!in_span(out, span[q])) out.push_back(span[q]);
-            for (int j = 0; j < N && (int)out.size() < k; ++j)
-                if (!in_span(out, 1ull << j)) out.push_back(1ull << j);
-            pp.out = out;
-            span.insert(span.end(), out.begin(), out.end());
-            if (rank_of(span) > D) return -3;
-        }
-        pp.end = e;
-        // independent basis of the span
-        std::vector<uint64_t> basis;
-        for (uint64_t v : span)
-            if (!in_span(basis, v)) basis.push_back(v);
-        pp.span = basis;
-        passes->push_back(pp);
-        I = pp.out;
-        s = e;
+        return v;
     }
-    return 0;
+    bool add(uint32_t v)
+    {
+        v = reduce(v);
+        if (!v) return false;
+        lead[31 - __builtin_clz(v)] = v;
+        ++dim;
+        return true;
+    }
+};
+
+// k vectors for the segments that a pass with span S writes and the next pass
+// reads: combinations of the next pass's stages U[e], U[e + 1], ... that lie in
+// S, the earliest first, so that they cost neither pass a dimension; `extra`
+// stage vectors that do not lie in S are taken as they come (they cost this
+// pass a dimension each).  What the stages do not give is filled from S.
+// Returns false if k vectors were not found.
+bool next_segments(const std::vector<uint64_t> &U, int e, int walk, int k, int extra,
+                   const Span &S, std::vector<uint32_t> *out)
+{
+    Span W = S;                     // S and the extra vectors taken
+    Span got;
+    uint32_t rest[32] = {}, comb[32] = {};  // stages outside W: reduced modulo W
+                                            // by leading bit, and the combination
+    out->clear();
+    for (int t = e; t < (int)U.size() && t < e + walk && (int)out->size() < k; ++t) {
+        const uint32_t u = (uint32_t)U[t];
+        uint32_t r = W.reduce(u), c = u;
+        while (r) {
+            const int b = 31 - __builtin_clz(r);
+            if (!rest[b]) break;
+            r = W.reduce(r ^ rest[b]);
+            c ^= comb[b];
+        }
+        if (!r) {
+            if (got.add(c)) out->push_back(c);
+        } else if (extra > 0) {
+            --extra;
+            W.add(u);
+            if (got.add(u)) out->push_back(u);
+            // the kept remainders modulo the larger W
+            uint32_t r0[32], c0[32];
+            memcpy(r0, rest, sizeof(r0));
+            memcpy(c0, comb, sizeof(c0));
+            memset(rest, 0, sizeof(rest));
+            for (int i = 0; i < 32; ++i) {
+                uint32_t r2 = W.reduce(r0[i]), c2 = c0[i];
+                while (r2) {
+                    const int b = 31 - __builtin_clz(r2);
+                    if (!rest[b]) {
+                        rest[b] = r2;
+                        comb[b] = c2;
+                        break;
+                    }
+                    r2 = W.reduce(r2 ^ rest[b]);
+                    c2 ^= comb[b];
+                }
+            }
+        } else {
+            rest[31 - __builtin_clz(r)] = r;
+            comb[31 - __builtin_clz(r)] = c;
+        }
+    }
+    for (int i = 0; i < 32 && (int)out->size() < k; ++i)
+        if (S.lead[i] && got.add(S.lead[i])) out->push_back(S.lead[i]);
+    return (int)out->size() == k;
 }
 
-// splitmix64, for the lane-vector search
-uint64_t mix64(uint64_t *s)
+// Stages from e on that fit a pass reading the segments in `in`.
+int stages_that_fit(const std::vector<uint64_t> &U, int e, const std::vector<uint32_t> &in, int D)
 {
-    uint64_t z = (*s += 0x9E3779B97F4A7C15ull);
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
+    Span sp;
+    for (uint32_t v : in) sp.add(v);
+    while (e < (int)U.size() && (sp.dim < D || !sp.reduce((uint32_t)U[e]))) {
+        sp.add((uint32_t)U[e]);
+        ++e;
+    }
+    return e;
+}
+
+// Cut the stages into passes (see above): a beam search over the cuts and the
+// segments between passes for the fewest passes.  A cut is (stages done,
+// segments); of the cuts reached with one pass more, those from which the next
+// pass gets furthest are kept.  Taking the most stages at every pass instead
+// leaves no dimension for the next pass's segments, which then cost that pass
+// k of its D: 29 passes at n = 24 (D = 14) where this finds 17, and 26 at
+// n = 20 (D = 12) where this finds 14.
+int group_stages(const std::vector<uint64_t> &U, int k, int D,
+                 const std::vector<uint64_t> &o_final, std::vector<PassPlan> *passes)
+{
+    constexpr int kBeam = 8;      // cuts kept per pass
+    constexpr int kShorter = 8;   // ends tried per cut: the furthest and earlier ones
+    const int S = (int)U.size();
+    struct Cut {
+        int from;                  // index of the cut before
+        int done;                  // stages run so far
+        int reach;                 // stages after one more pass
+        std::vector<uint32_t> in;  // segments the next pass reads
+    };
+    std::vector<Cut> cuts;  // every cut kept, in order of the passes
+    Cut first;
+    first.from = -1;
+    first.done = 0;
+    for (int j = 0; j < k; ++j) first.in.push_back(1u << j);
+    first.reach = stages_that_fit(U, 0, first.in, D);
+    cuts.push_back(first);
+    size_t begin = 0;
+    int last = -1;
+    while (last < 0) {
+        const size_t end = cuts.size();
+        std::vector<Cut> next;
+        for (size_t ci = begin; ci < end && last < 0; ++ci) {
+            const Cut &c = cuts[ci];
+            Span sp;
+            for (uint32_t v : c.in) sp.add(v);
+            std::vector<Span> spans;  // spans[i]: after stage c.done + i
+            int e = c.done;
+            while (e < S && e - c.done < kSortMaxStages &&
+                   (sp.dim < D || !sp.reduce((uint32_t)U[e]))) {
+                sp.add((uint32_t)U[e]);
+                spans.push_back(sp);
+                ++e;
+            }
+            if (e == S && !spans.empty()) {
+                // the last pass also writes the final layout's segments
+                Span all = sp;
+                for (uint64_t v : o_final) all.add((uint32_t)v);
+                if (all.dim <= D) {
+                    last = (int)ci;
+                    break;
+                }
+            }
+            const int low = e - kShorter > c.done ? e - kShorter : c.done;
+            for (int q = e; q > low; --q) {
+                if (q == S) continue;
+                const Span &s0 = spans[q - c.done - 1];
+                for (int extra = 0; extra <= D - s0.dim && extra <= k; ++extra) {
+                    Cut n;
+                    if (!next_segments(U, q, 4 * D, k, extra, s0, &n.in)) continue;
+                    n.from = (int)ci;
+                    n.done = q;
+                    n.reach = stages_that_fit(U, q, n.in, D);
+                    bool seen = false;
+                    for (const Cut &o : next) seen |= o.done == n.done && o.in == n.in;
+                    if (!seen) next.push_back(n);
+                }
+            }
+        }
+        if (last >= 0) break;
+        if (next.empty()) return -3;  // D too small to make progress
+        std::stable_sort(next.begin(), next.end(), [](const Cut &a, const Cut &b) {
+            return a.reach != b.reach ? a.reach > b.reach : a.done > b.done;
+        });
+        if ((int)next.size() > kBeam) next.resize(kBeam);
+        begin = end;
+        cuts.insert(cuts.end(), next.begin(), next.end());
+    }
+    // walk back from the last pass
+    std::vector<int> chain;
+    for (int ci = last; ci >= 0; ci = cuts[ci].from) chain.push_back(ci);
+    for (size_t i = chain.size(); i-- > 0;) {
+        const Cut &c = cuts[chain[i]];
+        PassPlan pp;
+        pp.first = c.done;
+        pp.end = i ? cuts[chain[i - 1]].done : S;
+        if (i)
+            pp.out.assign(cuts[chain[i - 1]].in.begin(), cuts[chain[i - 1]].in.end());
+        else
+            pp.out = o_final;
+        Span sp;
+        auto take = [&](uint64_t v) {
+            if (sp.add((uint32_t)v)) pp.span.push_back(v);
+        };
+        for (uint32_t v : c.in) take(v);
+        for (int q = pp.first; q < pp.end; ++q) take(U[q]);
+        for (uint64_t v : pp.out) take(v);
+        if (sp.dim > D) return -3;
+        passes->push_back(pp);
+    }
+    return 0;
 }
 
 // Basis of the vectors v of F2^P with parity(f & v) = 0 for every f in fs.
@@ -369,47 +484,30 @@ std::vector<uint64_t> nullspace(const std::vector<uint64_t> &fs, int P)
     return basis;
 }
 
-// Lanes for a group: 5 vectors of the span of `pool` whose low bank bits
-// (the 5 low slot bits for 4-byte keys, the 4 low ones of lanes 0-3 for
-// 8-byte keys) are independent, independent of `fixed` and of each other.
-// Falls back to the best rank found (bank conflicts, results still exact).
-bool pick_lanes(const std::vector<uint64_t> &pool, const std::vector<uint64_t> &fixed,
-                int e_log, uint64_t *seed, std::vector<uint64_t> *lanes)
+// Lanes for a group: 5 vectors of the pool (a basis of K0) whose low bank bits
+// (the 5 low slot bits for 4-byte keys, the 4 low ones of lanes 0-3 for 8-byte
+// keys) are as independent as the pool allows: elimination on the bank bits, the
+// vectors that keep one first.  With fewer, lanes share banks (results still
+// exact).  K0 meets the group's register vectors in 0, so any choice is
+// independent of those.
+// Returns the bank bits lost (0: conflict-free), or -1 for a pool too small.
+int pick_lanes(const std::vector<uint64_t> &pool, int e_log, std::vector<uint64_t> *lanes)
 {
-    const int bank_lanes = e_log == 2 ? 5 : 4;
-    const uint64_t bank_mask = e_log == 2 ? 31ull : 15ull;
-    int best = -1;
-    std::vector<uint64_t> best_lanes;
-    for (int tries = 0; tries < 4096; ++tries) {
-        std::vector<uint64_t> ln;
-        std::vector<uint64_t> all = fixed;
-        for (int t = 0; t < 5; ++t) {
-            uint64_t v = 0;
-            for (int attempt = 0; attempt < 64; ++attempt) {
-                v = 0;
-                const uint64_t pick = mix64(seed);
-                for (size_t i = 0; i < pool.size(); ++i)
-                    if ((pick >> (i % 64)) & 1ull) v ^= pool[i];
-                if (v && !in_span(all, v)) break;
-                v = 0;
-            }
-            if (!v) break;
-            ln.push_back(v);
-            all.push_back(v);
-        }
-        if (ln.size() != 5) continue;
-        std::vector<uint64_t> low;
-        for (int t = 0; t < bank_lanes; ++t) low.push_back(ln[t] & bank_mask);
-        const int r = rank_of(low);
-        if (r > best) {
-            best = r;
-            best_lanes = ln;
-        }
-        if (best == bank_lanes) break;
+    if (pool.size() < 5) return -1;
+    const int bank_bits = e_log == 2 ? 5 : 4;
+    std::vector<uint64_t> v = pool;
+    size_t r = 0;
+    for (int b = 0; b < bank_bits; ++b) {
+        size_t sel = r;
+        while (sel < v.size() && !((v[sel] >> b) & 1ull)) ++sel;
+        if (sel == v.size()) continue;
+        std::swap(v[r], v[sel]);
+        for (size_t i = 0; i < v.size(); ++i)
+            if (i != r && ((v[i] >> b) & 1ull)) v[i] ^= v[r];
+        ++r;
     }
-    if (best < 0) return false;
-    *lanes = best_lanes;
-    return true;
+    lanes->assign(v.begin(), v.begin() + 5);
+    return bank_bits - (int)r;
 }
 
 // Register groups of one pass and their thread mappings (physical slots).
@@ -417,17 +515,18 @@ bool pick_lanes(const std::vector<uint64_t> &pool, const std::vector<uint64_t> &
 // independent and the matrix M[a][b] = parity(hslot_a & delta_b) stays
 // invertible: then the common kernel K0 of the group's low tests is a
 // complement of the partner vectors, and the lanes, warps, rounds and unused
-// register bits are all taken from K0 (see SortStage).
+// register bits are all taken from K0 (see SortStage).  *conflicts receives the
+// extra shared-memory wavefronts of a key's round trips, over the groups.
 int build_groups(SortDesc *sd, const std::vector<uint32_t> &delta,
-                 const std::vector<uint32_t> &hslot, int P, int e_log)
+                 const std::vector<uint32_t> &hslot, int P, int e_log, int *conflicts)
 {
+    *conflicts = 0;
     const int R = kSortRegBits;
     const int round_bits = P - R - 8;
     if (round_bits < 0 || round_bits > kSortMaxRoundBits) return -3;
     sd->round_bits = (uint32_t)round_bits;
     const int S = (int)delta.size();
     int g = 0, s = 0;
-    uint64_t seed = 0xB17C0FFEEull ^ (uint64_t)P;
     auto m_invertible = [&](int first, int count) {
         std::vector<uint64_t> rows;
         for (int a = 0; a < count; ++a) {
@@ -455,7 +554,9 @@ int build_groups(SortDesc *sd, const std::vector<uint32_t> &delta,
         const std::vector<uint64_t> k0 = nullspace(fs, P);
         // lanes from K0, then unused register bits, warps and rounds from K0
         std::vector<uint64_t> lanes;
-        if (!pick_lanes(k0, reg, e_log, &seed, &lanes)) return -3;
+        const int lost = pick_lanes(k0, e_log, &lanes);
+        if (lost < 0) return -3;
+        *conflicts += (1 << lost) - 1;
         std::vector<uint64_t> all = reg;
         all.insert(all.end(), lanes.begin(), lanes.end());
         std::vector<uint64_t> fill;
@@ -501,6 +602,99 @@ int build_groups(SortDesc *sd, const std::vector<uint32_t> &delta,
     return 0;
 }
 
+// splitmix64, for the layout search
+uint64_t mix64(uint64_t *s)
+{
+    uint64_t z = (*s += 0x9E3779B97F4A7C15ull);
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+// Bank bits that a layout L takes from the low tests of the next pass's stages:
+// over runs of kSortRegBits stages, the low address bits (rows of L) that are
+// combinations of each other and of the run's tests.
+int bank_clashes(const PassPlan &next, const std::vector<uint64_t> &G, const f2::Mat &L, int e_log)
+{
+    const int bank_bits = e_log == 2 ? 5 : 4;
+    int clashes = 0;
+    for (int s = next.first; s < next.end; s += kSortRegBits) {
+        Span sp;
+        for (int q = s; q < next.end && q < s + kSortRegBits; ++q) sp.add((uint32_t)G[q]);
+        for (int i = 0; i < bank_bits; ++i) clashes += !sp.add((uint32_t)L.r[i]);
+    }
+    return clashes;
+}
+
+// Tables of one pass from layout L_prev to layout L.  *score receives the extra
+// shared-memory wavefronts of its register groups and stores.
+int derive_sort_pass(const PassPlan &pp, const std::vector<uint64_t> &U,
+                     const std::vector<uint64_t> &G, const f2::Mat &L, const f2::Mat &L_prev,
+                     const f2::Mat &L_prev_inv, int N, int e_log, int key, int k, int D,
+                     int compare_code, PassDesc *desc_out, SortDesc *sd_out, int *score)
+{
+    PassDesc &desc = *desc_out;
+    const f2::Mat T = f2::mul(L, L_prev_inv);
+    // the block span in physical input positions, padded with unit
+    // vectors up to D dimensions
+    std::vector<uint64_t> W;
+    for (uint64_t v : pp.span) W.push_back(L_prev.apply(v));
+    for (int j = 0; j < N && rank_of(W) < D; ++j)
+        if (!in_span(W, 1ull << j)) W.push_back(1ull << j);
+    PassInfo info;
+    SlotMap map;
+    PlanOptions opt;
+    opt.seg_bits = k;
+    int rc = derive_pass_span(T, 0, N, e_log, opt, W.data(), (int)W.size(), &desc, &info, &map);
+    if (rc) return rc;
+    if (desc.naive || map.P != D || desc.thread_bits != 8) return BMMC_ERR_UNSUPPORTED;
+    std::vector<uint64_t> lam(map.lam, map.lam + map.P);
+
+    SortDesc &sd = *sd_out;
+    memset(&sd, 0, sizeof(sd));
+    sd.key = (uint32_t)key;
+    // The unrolled orientation variants pay off on large arrays of 4-byte
+    // keys (GB300: 5 % at 2^20, 11 % at 2^22 and 2^24); smaller sorts are
+    // bound by latency, where the compact loop's smaller code fetches
+    // faster, and 8-byte keys measured faster with the compact loop at
+    // every size.
+    sd.unrolled = compare_code == 2 ||
+                  (compare_code == 0 && e_log == 2 && N >= kSortUnrolledMinBits);
+    sd.n_stage = (uint32_t)(pp.end - pp.first);
+    std::vector<uint32_t> delta, hslot;
+    for (int s = pp.first; s < pp.end; ++s) {
+        const uint64_t v = L_prev.apply(U[s]);
+        uint64_t coords = 0;
+        if (!solve(lam, v, &coords)) return BMMC_ERR_INVALID;
+        const uint32_t dl = map.swz((uint32_t)coords);
+        // g_s . x_virtual = g_s . (L_prev^{-1} x_physical)
+        uint64_t hin = 0;
+        for (int j = 0; j < N; ++j)
+            hin |= (uint64_t)__builtin_parityll(G[s] & L_prev_inv.col(j)) << j;
+        uint32_t hs = 0;
+        for (int i = 0; i < map.P; ++i) {
+            const uint64_t off = xor_bits64(lam.data(), map.swz(1u << i));
+            hs |= (uint32_t)__builtin_parityll(hin & off) << i;
+        }
+        if (!__builtin_parity(hs & dl)) return BMMC_ERR_INVALID;  // g_s . u_s = 1
+        SortStage &st = sd.st[s - pp.first];
+        st.hin = (uint32_t)hin;
+        delta.push_back(dl);
+        hslot.push_back(hs);
+    }
+    for (uint32_t bb = 0; bb < desc.n_cta; ++bb) {
+        uint64_t m = 0;
+        for (int s = pp.first; s < pp.end; ++s)
+            m |= (uint64_t)__builtin_parity(sd.st[s - pp.first].hin & desc.cta_in[bb])
+                 << (s - pp.first);
+        sd.cta_mask[bb] = m;
+    }
+    rc = build_groups(&sd, delta, hslot, map.P, e_log, score);
+    if (rc) return rc;
+    *score += info.wavefronts_store - info.ideal_store;
+    return BMMC_OK;
+}
+
 }  // namespace
 
 int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int compare_code)
@@ -544,7 +738,9 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int co
         return BMMC_OK;
     }
 
-    const int k = default_seg_bits(e_log);
+    // Segments of one 128-byte line: each of their bits costs a pass that reads
+    // or writes them a dimension of its block.
+    const int k = 7 - e_log;
     // Default block: 64 KiB (more stages per pass), but small enough that a
     // pass has at least 512 thread blocks to spread over the SMs, and at
     // least 2^12 keys.
@@ -563,86 +759,59 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int co
     for (int j = 0; j < k; ++j) o_final.push_back(qfin_inv.col(j));
 
     std::vector<PassPlan> plans;
-    int rc = group_stages(U, N, k, D, o_final, &plans);
+    int rc = group_stages(U, k, D, o_final, &plans);
     if (rc) return rc;
 
     f2::Mat L_prev = f2::Mat::identity(N), L_prev_inv = f2::Mat::identity(N);
+    uint64_t seed = 0xB17C0FFEEull;
     for (size_t pi = 0; pi < plans.size(); ++pi) {
         const PassPlan &pp = plans[pi];
         const bool last = pi + 1 == plans.size();
-        f2::Mat L, L_inv;
-        if (last) {
-            L = qfin;
-            L_inv = qfin_inv;
-        } else {
-            std::vector<uint64_t> cols = pp.out;
-            for (int j = 0; j < N && (int)cols.size() < N; ++j)
-                if (!in_span(cols, 1ull << j)) cols.push_back(1ull << j);
-            L_inv = from_columns(cols, N);
-            if (!f2::inverse(L_inv, &L)) return BMMC_ERR_INVALID;
-        }
-        const f2::Mat T = f2::mul(L, L_prev_inv);
-        // the block span in physical input positions, padded with unit
-        // vectors up to D dimensions
-        std::vector<uint64_t> W;
-        for (uint64_t v : pp.span) W.push_back(L_prev.apply(v));
-        for (int j = 0; j < N && rank_of(W) < D; ++j)
-            if (!in_span(W, 1ull << j)) W.push_back(1ull << j);
-        PassDesc desc;
-        PassInfo info;
-        SlotMap map;
-        PlanOptions opt;
-        rc = derive_pass_span(T, 0, N, e_log, opt, W.data(), (int)W.size(), &desc, &info, &map);
-        if (rc) return rc;
-        if (desc.naive || map.P != D || desc.thread_bits != 8) return BMMC_ERR_UNSUPPORTED;
-        std::vector<uint64_t> lam(map.lam, map.lam + map.P);
-
-        SortDesc sd;
-        memset(&sd, 0, sizeof(sd));
-        sd.key = (uint32_t)key;
-        // The unrolled orientation variants pay off on large arrays of 4-byte
-        // keys (GB300: 5 % at 2^20, 11 % at 2^22 and 2^24); smaller sorts are
-        // bound by latency, where the compact loop's smaller code fetches
-        // faster, and 8-byte keys measured faster with the compact loop at
-        // every size.
-        sd.unrolled = compare_code == 2 ||
-                      (compare_code == 0 && e_log == 2 && N >= kSortUnrolledMinBits);
-        sd.n_stage = (uint32_t)(pp.end - pp.first);
-        std::vector<uint32_t> delta, hslot;
-        for (int s = pp.first; s < pp.end; ++s) {
-            const uint64_t v = L_prev.apply(U[s]);
-            uint64_t coords = 0;
-            if (!solve(lam, v, &coords)) return BMMC_ERR_INVALID;
-            const uint32_t dl = map.swz((uint32_t)coords);
-            // g_s . x_virtual = g_s . (L_prev^{-1} x_physical)
-            uint64_t hin = 0;
-            for (int j = 0; j < N; ++j)
-                hin |= (uint64_t)__builtin_parityll(G[s] & L_prev_inv.col(j)) << j;
-            uint32_t hs = 0;
-            for (int i = 0; i < map.P; ++i) {
-                const uint64_t off = xor_bits64(lam.data(), map.swz(1u << i));
-                hs |= (uint32_t)__builtin_parityll(hin & off) << i;
+        // A layout between passes is free outside its segments: each other basis
+        // vector may have any segment vector added.  That changes which
+        // functionals the low address bits are, and so which keys share a
+        // shared-memory bank: where a low test g_s of a register group is a
+        // combination of the bank bits, no choice of lanes avoids conflicts.
+        // The vectors as they come leave half of the tests so in the passes that
+        // start at the network's first stages; a few tries of random additions
+        // find layouts with none or nearly none (n = 24 float32, the 17 passes:
+        // 1482 us with the vectors as they come, 1161 us so).
+        constexpr int kTries = 6;
+        int best = -1;
+        for (int attempt = 0; attempt < (last ? 1 : kTries) && best != 0; ++attempt) {
+            f2::Mat L, L_inv;
+            if (last) {
+                L = qfin;
+                L_inv = qfin_inv;
+            } else {
+                std::vector<uint64_t> cols = pp.out;
+                for (int j = 0; j < N && (int)cols.size() < N; ++j)
+                    if (!in_span(cols, 1ull << j)) cols.push_back(1ull << j);
+                if (attempt)
+                    for (int j = k; j < N; ++j) cols[j] ^= xor_bits64(cols.data(), mix64(&seed) >> (64 - k));
+                L_inv = from_columns(cols, N);
+                if (!f2::inverse(L_inv, &L)) return BMMC_ERR_INVALID;
             }
-            if (!__builtin_parity(hs & dl)) return BMMC_ERR_INVALID;  // g_s . u_s = 1
-            SortStage &st = sd.st[s - pp.first];
-            st.hin = (uint32_t)hin;
-            delta.push_back(dl);
-            hslot.push_back(hs);
+            PassDesc desc;
+            SortDesc sd;
+            int score = 0;
+            rc = derive_sort_pass(pp, U, G, L, L_prev, L_prev_inv, N, e_log, key, k, D,
+                                  compare_code, &desc, &sd, &score);
+            if (rc) return rc;
+            if (!last) score += bank_clashes(plans[pi + 1], G, L, e_log);
+            if (best >= 0 && score >= best) continue;
+            if (best >= 0) {
+                p->pass.pop_back();
+                p->ce.pop_back();
+                p->layout.pop_back();
+            }
+            best = score;
+            p->pass.push_back(desc);
+            p->ce.push_back(sd);
+            p->layout.push_back(L);
         }
-        for (uint32_t bb = 0; bb < desc.n_cta; ++bb) {
-            uint64_t m = 0;
-            for (int s = pp.first; s < pp.end; ++s)
-                m |= (uint64_t)__builtin_parity(sd.st[s - pp.first].hin & desc.cta_in[bb])
-                     << (s - pp.first);
-            sd.cta_mask[bb] = m;
-        }
-        rc = build_groups(&sd, delta, hslot, map.P, e_log);
-        if (rc) return rc;
-        p->pass.push_back(desc);
-        p->ce.push_back(sd);
-        p->layout.push_back(L);
-        L_prev = L;
-        L_prev_inv = L_inv;
+        L_prev = p->layout.back();
+        f2::inverse(L_prev, &L_prev_inv);
     }
     return BMMC_OK;
 }
