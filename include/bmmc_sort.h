@@ -33,15 +33,12 @@ extern "C" {
 typedef struct bmmc_sort_plan_s *bmmc_sort_plan;
 
 typedef struct bmmc_sort_options {
-    int block_log2;   /* log2 of the bytes one thread block holds; 0 = up to
-                         64 KiB, smaller for arrays that would give a pass
-                         fewer than 512 thread blocks.  Must leave room for
-                         2^12 keys and be at most 64 KiB. */
-    int compare_code; /* how a thread block runs its comparators: 0 = by
-                         block size, 1 = one compact loop (less code: faster
-                         for small, latency-bound sorts), 2 = a variant per
-                         comparator orientation (fewer instructions: faster
-                         for large sorts).  Same results either way. */
+    int block_log2;   /* log2 of the bytes one thread block holds; 0 = 16 to
+                         64 KiB by the size of the array.  Must leave room for
+                         2^12 keys and be at most 64 KiB; arrays of at most
+                         2^12 keys are one block whatever it is. */
+    int compare_code; /* 0, 1 or 2; the comparators have one form, and the
+                         value makes no difference. */
     int reserved[6];  /* must be zero */
 } bmmc_sort_options;
 

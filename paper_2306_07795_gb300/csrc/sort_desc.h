@@ -12,68 +12,86 @@
 // into shared memory, a block runs those stages on it and only then writes
 // it out, in the layout the next pass reads.
 //
-// Inside a pass the stages are cut into groups of at most R stages.  For one
-// group every thread holds 2^R elements in registers: slot (physical, element
-// units) = thread part + round part + reg_off(j), j < 2^R, with reg_off linear
-// in the bits of j.  The k-th stage of a group pairs the slots that differ in
-// register bit k (its partner vector is the group's k-th register vector), so
-// a stage is a compare-exchange between two registers of one thread, and the
-// kernel runs the k-th stage with register bit k fixed at compile time.
+// Inside a pass the stages are cut into groups.  The f <= R distinct low tests
+// of a group's stages, in the order of the network's index bits, are the first
+// coordinates of the 2^R keys that a thread holds in registers for the group:
+// register j holds the key whose index has test t equal to bit t of j, for
+// every t < f, in every thread and block.  The planner finds the slot vectors
+// reg[t] dual to the tests in the span of the partner vectors, takes lanes,
+// warps and the unused register bits from the common kernel of the tests, and
+// moves the block's own part of the tests into its slot base (cta).  So a
+// stage is the same exchange between registers everywhere: it pairs j with
+// j ^ m, where m, the partner vector in the tests' coordinates, turns out to
+// be a run of ones from bit i (the stage's own test) to bit l - 1, and the
+// register with bit i clear takes the smaller key.  There are R (R + 1) / 2
+// such stages, compiled as that many variants, against 2 R 2^(R-1) with
+// registers in the order of the partner vectors, where the test is a parity of
+// several register bits and of the block.  A group may hold more than R
+// stages: the network's first R levels are one group of R (R + 1) / 2.
 // Between groups the registers go back to shared memory.
 #pragma once
 #include <stdint.h>
 
+#include "pass_desc.h"
+
 namespace bmmc {
 
-constexpr int kSortRegBits = 4;          // R: 16 registers per round
-constexpr int kSortMaxStages = 64;       // stages in one pass
-constexpr int kSortMaxGroups = 40;       // register groups in one pass
-constexpr int kSortMaxRoundBits = 6;     // rounds per group = 2^round_bits
-constexpr int kSortSmallMaxBits = 12;    // one-block sort: at most 2^12 keys
-constexpr int kSortSmallMaxStages = 78;  // 12 * 13 / 2
-constexpr int kSortUnrolledMinBits = 20; // unrolled compares from 2^20 4-byte keys
+constexpr int kSortMaxRegBits = 5;     // R: at most 32 keys per thread
+constexpr int kSortMaxThreadBits = 8;  // 256 threads
+constexpr int kSortMaxGroups = 26;     // register groups in one pass
+constexpr int kSortMaxGroupStages = 16;
+constexpr int kSortMaxCtaBits = 20;    // thread-block bits: 32 - 12
+constexpr int kSortSmallMaxBits = 7;   // bmmc_sort_small: at most 2^7 keys
+constexpr int kSortSmallMaxStages = 28;  // 7 * 8 / 2
 
-// The low test of a stage: the element at physical slot q of the block
-// whose input base is x_b takes the smaller key of its pair iff
-// parity(hin & x_b) + parity(hslot & q) = 0.  The planner puts every lane,
-// warp and round vector of the stage's group in the kernel of hslot, so the
-// slot part depends only on the register index j: parity(hslot & reg_off(j))
-// = parity(j & hmask) for the j whose stage bit is 0.  Register j of every
-// thread of the block is thus the low one iff parity(j & hmask) equals the
-// block's bit parity(hin & x_b): one orientation pattern per block and
-// stage, known without any per-thread test.
-struct SortStage {
-    uint32_t hin;    // input part of the low test
-    uint16_t low0;   // bit j: register j is the low position when the block's
-                     // bit is 0 (parity(j & hmask) = 0); the complement when 1
-    uint8_t hmask;   // register bits t != k with parity(hslot & reg[t]) = 1
-    uint8_t pad;
-};
+// The stage pairing register j with j ^ (ones at bits i..l-1), bit i low.
+constexpr BMMC_HD int sort_stage_code(int i, int l) { return l * (l - 1) / 2 + i; }
 
 struct SortGroup {
-    uint16_t first, count;          // stages [first, first + count), count <= R
-    uint16_t reg[kSortRegBits];     // slot vector of register bit t
-    uint16_t lane[5];               // slot vector of lane bit t
-    uint16_t warp[3];               // slot vector of warp bit t
-    uint16_t round[kSortMaxRoundBits];  // slot vector of round bit t
+    uint16_t n_stage;                // stages of the group
+    uint16_t reg[kSortMaxRegBits];   // slot vector of register bit t
+    uint32_t code[2];                // sort_stage_code of stage s: 4 bits at 4 s
+    uint16_t lane[5];                // slot vector of lane bit t
+    uint16_t warp[kSortMaxThreadBits - 5];  // slot vector of warp bit t
+    uint16_t round;                  // slot vector of the second round
+    uint16_t cta[kSortMaxCtaBits];   // slot part of thread-block bit b
+    uint16_t pad;
+};
+
+// How the 16-byte chunks of a tile come in and go out (the tables of pass_desc.h
+// by chunk bits of this kernel's blocks): chunk c of a thread, for the input
+// its place in the array and in the tile, for the output the tile offset of its
+// first element and its place in the array, each the XOR of the entries of the
+// set bits of (thread block, warp, lane, c).
+enum SortField { kSortIn = 0, kSortDst = 1, kSortSrc = 2, kSortOut = 3 };
+
+struct SortTile {
+    // thread-block bits, then warp bits; in and out in elements, tile in bytes
+    uint32_t block[4][kSortMaxCtaBits + kSortMaxThreadBits - 5];
+    uint32_t lane[4][5];
+    uint32_t chunk[4][4];
+    uint32_t elem[4];  // tile offset of element j of an output chunk
+    uint32_t rot[5];   // element rotation of a lane bit: load j gives element j ^ rot
+    uint32_t any_rot;
 };
 
 struct SortDesc {
     uint32_t key;          // bmmc_key_type of the keys
-    uint32_t unrolled;     // 1: each stage runs a variant with its orientation
-                           //    fixed at compile time (3 instructions per pair,
-                           //    more code); 0: one loop reading low0 (6 per pair)
+    uint32_t reg_bits;     // R
+    uint32_t rounds;       // 1 or 2: sets of 2^R keys that a thread runs in turn
     uint32_t n_stage;
+    uint32_t n_cta;        // 2^n_cta thread blocks
+    uint32_t tile_bytes;   // bytes of a tile, 2^(P + e_log)
+    uint32_t first_pass;   // 1: reads the caller's keys; between passes 8-byte
+    uint32_t last_pass;    //    float keys are kept as ordered integers
     uint32_t n_group;
-    uint32_t round_bits;   // rounds per group = 2^round_bits
-    uint64_t cta_mask[32]; // per thread-block bit b: bit s = parity(hin_s & cta_in[b])
-    SortStage st[kSortMaxStages];
+    SortTile tile;
     SortGroup grp[kSortMaxGroups];
 };
 
-// The whole network on one thread block, for arrays of at most 2^12 keys:
-// the keys stay in shared memory at their virtual positions, and the block
-// writes key x to out[fin x] at the end.
+// The whole network on one thread block, for arrays of at most 2^7 keys: the
+// keys stay in shared memory at their virtual positions, and the block writes
+// key x to out[fin x] at the end.
 struct SortSmallDesc {
     uint32_t N;        // 2^N keys
     uint32_t key;

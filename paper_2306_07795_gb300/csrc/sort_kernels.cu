@@ -4,16 +4,17 @@
 // shared memory, barrier, 16-byte gathers and stores: dev::tile_load and
 // dev::tile_store of tile_body.cuh) with comparator stages run on the tile in
 // between.  The stages come in groups (sort_desc.h): for one group, every
-// thread loads 16 keys of the tile into registers per round, and each stage
-// of the group orders pairs of those registers, the pair's low position
-// (index with g_s . x = 0) receiving the smaller key (Sec. 6.1: a pair is
-// kept when first <= second and swapped otherwise).  The keys go back to the
-// same slots, and a barrier separates the groups.
+// thread loads 2^R keys of the tile into registers, and each stage of the group
+// orders pairs of those registers, the pair's low position (index with
+// g_s . x = 0) receiving the smaller key (Sec. 6.1: a pair is kept when
+// first <= second and swapped otherwise).  The keys go back to the same slots,
+// and a barrier separates the groups.
 //
-// Arrays of at most 2^12 keys run the whole network in one thread block
-// (bmmc_sort_small): keys at their positions in shared memory, one stage at a
-// time, then each key to its final position.
+// Arrays of at most 2^12 keys are one block of that kernel; those of at most
+// 2^7 run in bmmc_sort_small: keys at their positions in shared memory, one
+// stage at a time, then each key to its final position.
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <atomic>
@@ -30,29 +31,6 @@ template <int E_LOG> struct KeyWord;
 template <> struct KeyWord<2> { using type = uint32_t; };
 template <> struct KeyWord<3> { using type = unsigned long long; };
 
-template <int E_LOG>
-__device__ __forceinline__ typename KeyWord<E_LOG>::type lds_key(uint32_t addr)
-{
-    if constexpr (E_LOG == 2) {
-        uint32_t v;
-        asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(v) : "r"(addr));
-        return v;
-    } else {
-        unsigned long long v;
-        asm volatile("ld.shared.b64 %0, [%1];\n" : "=l"(v) : "r"(addr));
-        return v;
-    }
-}
-
-template <int E_LOG>
-__device__ __forceinline__ void sts_key(uint32_t addr, typename KeyWord<E_LOG>::type v)
-{
-    if constexpr (E_LOG == 2)
-        asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
-    else
-        asm volatile("st.shared.b64 [%0], %1;\n" ::"r"(addr), "l"(v) : "memory");
-}
-
 // Sec. 6.1's comparator: the pair (a at the low position, b at the high one)
 // is kept when a <= b.
 template <int KEY, typename V>
@@ -62,215 +40,437 @@ __device__ __forceinline__ bool keep(V a, V b)
     else return dev::keep_pair64<KEY>((uint64_t)a, (uint64_t)b);
 }
 
-// The register sets of a thread: NR independent rounds of 2^kSortRegBits
-// keys each, compared in the same stages (their orientation is the same:
-// it depends on the register index and the block only), so that the
-// compare-exchanges of one set fill the latency of the other's.
-template <typename V, int NR>
-using RegSets = V[NR][1 << kSortRegBits];
-
-// One stage on the registers, compact form: the pairs (j, j + 2^I); bit j
-// of `low` tells whether register j is the pair's low position.  Six
-// instructions per pair.
-template <int I, int KEY, int NR, typename V>
-__device__ __forceinline__ void ce_regs(RegSets<V, NR> &v, uint32_t low)
+// Float keys without NaN and -0.0 are totally ordered, and the pair may be
+// ordered by other means than IEEE <=: 4-byte ones by minimum and maximum, and
+// 8-byte ones, whose compare runs on the FP64 pipe at about two lanes a clock
+// per SM, as integers of the same order.  A block looks at its keys as it
+// first loads them and uses <= itself for the whole pass if any is special.
+//
+// ordered(): the integer of a double's order, and back (its own inverse); the
+// order of signed integers is that of <= outside special keys, NaN beyond the
+// infinities and -0.0 just below +0.0.
+__device__ __forceinline__ unsigned long long ordered(unsigned long long x)
 {
+    const uint32_t hi = (uint32_t)(x >> 32), m = (uint32_t)((int32_t)hi >> 31);
+    return ((unsigned long long)(hi ^ (m & 0x7fffffffu)) << 32) | ((uint32_t)x ^ m);
+}
+
+// NaN or -0.0 (8-byte keys as ordered() gives them; there also the infinities
+// and negative numbers too small for the high word).
+template <int KEY>
+__device__ __forceinline__ bool special(uint32_t x)
+{
+    return !(__uint_as_float(x) == __uint_as_float(x)) || x == 0x80000000u;
+}
+template <int KEY>
+__device__ __forceinline__ bool special(unsigned long long x)
+{
+    const uint32_t hi = (uint32_t)(x >> 32);
+    return hi - 0x80100000u >= 0x7ff00000u - 0x80100000u || hi == ~0u;
+}
+
+// How a stage orders pairs: as the key type, or one of these.
+constexpr int kF32MinMax = 7;   // 4-byte float keys, none special
+constexpr int kF64Ordered = 8;  // ordered() 8-byte float keys, compared as doubles
+
+// Runtime 1 and -1 (from a kernel parameter, so that the compiler keeps the
+// products): x * one + y and y - x as 32-bit multiply-adds.
+struct Units {
+    uint32_t one, minus_one;
+};
+
+__device__ __forceinline__ uint32_t mad32(uint32_t x, uint32_t m, uint32_t y)
+{
+    uint32_t r;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(m), "r"(y));
+    return r;
+}
+
+// The other one of the pair {a, b}, given one of them: a + b - x.
+__device__ __forceinline__ uint32_t other(uint32_t a, uint32_t b, uint32_t x, Units u)
+{
+    return mad32(x, u.minus_one, mad32(a, u.one, b));
+}
+__device__ __forceinline__ unsigned long long other(unsigned long long a, unsigned long long b,
+                                                    unsigned long long x, Units u)
+{
+    // word by word: both words of x come from the same key
+    const uint32_t lo = other((uint32_t)a, (uint32_t)b, (uint32_t)x, u);
+    const uint32_t hi =
+        other((uint32_t)(a >> 32), (uint32_t)(b >> 32), (uint32_t)(x >> 32), u);
+    return ((unsigned long long)hi << 32) | lo;
+}
+
+// How many pairs of four take their other key from multiply-adds: the compares,
+// minima and selects of a pair run on the ALU pipe at half the issue rate, and
+// sharing the work with the multiply-add pipe is faster.  n = 24, none / two /
+// three / all of four, us: int32 769 / 742 / 747 / 753, float32 830 / 801 / 811 /
+// 811, int64 1991 / 1814 / 1717 / 1673, float64 2198 / 2008 / 1926 / 1913.
+template <typename V> constexpr int kMadPairs = sizeof(V) == 4 ? 2 : 4;
+
+// Order the pair: a becomes the low one, b the high one.
+template <int HOW, bool MAD>
+__device__ __forceinline__ void order(uint32_t &a, uint32_t &b, Units u)
+{
+    uint32_t lo, hi;
+    if constexpr (HOW == kF32MinMax) {
+        lo = __float_as_uint(fminf(__uint_as_float(a), __uint_as_float(b)));
+        hi = __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
+    } else {
+        const bool k = keep<HOW>(a, b);
+        lo = k ? a : b;
+        hi = k ? b : a;
+    }
+    if constexpr (MAD) hi = other(a, b, lo, u);
+    a = lo;
+    b = hi;
+}
+template <int HOW, bool MAD>
+__device__ __forceinline__ void order(unsigned long long &a, unsigned long long &b, Units u)
+{
+    bool k;
+    if constexpr (HOW == kF64Ordered) k = keep<dev::kKeyF64>(ordered(a), ordered(b));
+    else k = keep<HOW>(a, b);
+    const unsigned long long lo = k ? a : b;
+    b = MAD ? other(a, b, lo, u) : k ? b : a;
+    a = lo;
+}
+
+// One stage on the registers: the pairs (j, j ^ ones at bits I..L-1), bit I of j
+// clear at the low position.
+template <int I, int L, int HOW, int R, int J = 0, typename V>
+__device__ __forceinline__ void ce_run(V (&v)[1 << R], Units u)
+{
+    if constexpr (L <= R && J < (1 << R)) {
+        constexpr int nth = (J & ((1 << I) - 1)) | ((J >> (I + 1)) << I);
+        if constexpr (!(J & (1 << I)))
+            order<HOW, ((nth & 3) < kMadPairs<V>)>(v[J], v[J ^ ((1 << L) - (1 << I))], u);
+        ce_run<I, L, HOW, R, J + 1>(v, u);
+    }
+}
+
+// The stage of a sort_stage_code (the same for the whole block).
+template <int HOW, int R, typename V>
+__device__ __forceinline__ void ce_stage(uint32_t code, V (&v)[1 << R], Units u)
+{
+    static_assert(kSortMaxRegBits == 5, "one case per stage code");
+    switch (code) {
+    case sort_stage_code(0, 1): ce_run<0, 1, HOW, R>(v, u); break;
+    case sort_stage_code(0, 2): ce_run<0, 2, HOW, R>(v, u); break;
+    case sort_stage_code(1, 2): ce_run<1, 2, HOW, R>(v, u); break;
+    case sort_stage_code(0, 3): ce_run<0, 3, HOW, R>(v, u); break;
+    case sort_stage_code(1, 3): ce_run<1, 3, HOW, R>(v, u); break;
+    case sort_stage_code(2, 3): ce_run<2, 3, HOW, R>(v, u); break;
+    case sort_stage_code(0, 4): ce_run<0, 4, HOW, R>(v, u); break;
+    case sort_stage_code(1, 4): ce_run<1, 4, HOW, R>(v, u); break;
+    case sort_stage_code(2, 4): ce_run<2, 4, HOW, R>(v, u); break;
+    case sort_stage_code(3, 4): ce_run<3, 4, HOW, R>(v, u); break;
+    case sort_stage_code(0, 5): ce_run<0, 5, HOW, R>(v, u); break;
+    case sort_stage_code(1, 5): ce_run<1, 5, HOW, R>(v, u); break;
+    case sort_stage_code(2, 5): ce_run<2, 5, HOW, R>(v, u); break;
+    case sort_stage_code(3, 5): ce_run<3, 5, HOW, R>(v, u); break;
+    case sort_stage_code(4, 5): ce_run<4, 5, HOW, R>(v, u); break;
+    }
+}
+
+// The stages of a group.
+template <int HOW, int R, typename V>
+__device__ __forceinline__ void run_stages(uint32_t n_stage, uint64_t codes, V (&v)[1 << R], Units u)
+{
+    for (uint32_t s = n_stage; s > 0; --s, codes >>= 4)
+        ce_stage<HOW, R>((uint32_t)codes & 15u, v, u);
+}
+
+// XOR of tab[b] over the set bits b of v, b < N.
+template <int N>
+__device__ __forceinline__ uint32_t xor_table(const uint16_t *tab, uint32_t v)
+{
+    uint32_t acc = 0;
 #pragma unroll
-    for (int j = 0; j < (1 << kSortRegBits); ++j) {
-        if (j & (1 << I)) continue;
-        constexpr int bit = 1 << I;
-        const bool lj = (low >> j) & 1u;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const V a = v[r][j], b = v[r][j | bit];
-            const bool k = lj ? keep<KEY>(a, b) : keep<KEY>(b, a);
-            v[r][j] = k ? a : b;
-            v[r][j | bit] = k ? b : a;
+    for (int b = 0; b < N; ++b)
+        if ((v >> b) & 1u) acc ^= tab[b];
+    return acc;
+}
+
+// What a block keeps in shared memory behind its tile: the pass's tables, and
+// for each group, in bytes, what its threads read: codes and register offsets in
+// a few words, offsets of its lanes (the block's own part included) and warps.
+struct GroupTab {
+    uint4 head;      // codes; register offsets 0 | 1 << 16, 2 | 3 << 16
+    uint32_t reg4;   // register offset 4 | stages << 16
+    uint32_t round;
+    uint16_t lane[32];
+    uint16_t warp[1 << (kSortMaxThreadBits - 5)];
+    uint32_t pad[2];
+};
+struct SortTab {
+    GroupTab grp[kSortMaxGroups];
+    SortDesc d;
+};
+
+// Fill tab.grp, a warp per group.
+template <int E_LOG>
+__device__ __forceinline__ void expand_groups(SortTab &tab, uint32_t cta, uint32_t n_cta)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const bool cta_bit = lane < n_cta && ((cta >> lane) & 1u);
+    for (uint32_t gi = threadIdx.x >> 5; gi < tab.d.n_group; gi += blockDim.x >> 5) {
+        const SortGroup &G = tab.d.grp[gi];
+        GroupTab &g = tab.grp[gi];
+        const uint32_t base = __reduce_xor_sync(0xffffffffu, cta_bit ? (uint32_t)G.cta[lane] : 0u);
+        g.lane[lane] = (uint16_t)((base ^ xor_table<5>(G.lane, lane)) << E_LOG);
+        if (lane < (1u << (kSortMaxThreadBits - 5)))
+            g.warp[lane] = (uint16_t)(xor_table<kSortMaxThreadBits - 5>(G.warp, lane) << E_LOG);
+        if (lane == 31u) {
+            g.head = make_uint4(G.code[0], G.code[1],
+                                ((uint32_t)G.reg[0] | (uint32_t)G.reg[1] << 16) << E_LOG,
+                                ((uint32_t)G.reg[2] | (uint32_t)G.reg[3] << 16) << E_LOG);
+            g.reg4 = (uint32_t)G.reg[4] << E_LOG | (uint32_t)G.n_stage << 16;
+            g.round = (uint32_t)G.round << E_LOG;
         }
     }
 }
 
-template <int KEY, int NR, typename V>
-__device__ __forceinline__ void ce_regs_k(int k, RegSets<V, NR> &v, uint32_t low)
-{
-    if (k == 0) ce_regs<0, KEY, NR>(v, low);
-    else if (k == 1) ce_regs<1, KEY, NR>(v, low);
-    else if (k == 2) ce_regs<2, KEY, NR>(v, low);
-    else ce_regs<3, KEY, NR>(v, low);
-}
+// Byte offset of register j of a group: off[j % 8] ^ top[j / 8].
+template <int R>
+struct RegOffsets {
+    static constexpr int LO = 8, HI = (1 << R) / LO;
+    uint32_t off[LO], top[HI];
 
-// One stage on the registers with its orientation fixed at compile time:
-// the pairs (j, j + 2^K), and register j is the pair's low position (it
-// keeps the smaller key, Sec. 6.1) iff parity(j & HM) == B.  Three
-// instructions per pair: one comparison, two selects.
-template <int K, int HM, int B, int KEY, int NR, typename V>
-__device__ __forceinline__ void ce_fixed(RegSets<V, NR> &v)
-{
+    // reg: byte offsets of the register bits, two in a word
+    __device__ __forceinline__ RegOffsets(const uint32_t (&reg)[3], uint32_t base)
+    {
+        off[0] = base;
+        top[0] = 0;
 #pragma unroll
-    for (int j = 0; j < (1 << kSortRegBits); ++j) {
-        if (j & (1 << K)) continue;
-        const int jj = j | (1 << K);
-        const bool low = (__popc(j & HM) & 1) == B;
-        const int lo = low ? j : jj, hi = low ? jj : j;
+        for (int t = 0; t < R; ++t) {
+            const uint32_t v = t & 1 ? reg[t / 2] >> 16 : reg[t / 2] & 0xffffu;
+            if (t < 3) {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const V a = v[r][lo], b = v[r][hi];
-            const bool k = keep<KEY>(a, b);
-            v[r][lo] = k ? a : b;
-            v[r][hi] = k ? b : a;
-        }
-    }
-}
-
-// Select the variant of stage bit K for the block's (hm, b): hm has bit K
-// clear; both are the same for every thread of the block.
-template <int K, int KEY, int HM, int NR, typename V>
-__device__ __forceinline__ void ce_dispatch(RegSets<V, NR> &v, uint32_t hm, uint32_t b)
-{
-    if constexpr (HM < (1 << kSortRegBits)) {
-        if constexpr ((HM >> K) & 1) {
-            ce_dispatch<K, KEY, HM + 1, NR>(v, hm, b);
-        } else {
-            if (hm == (uint32_t)HM) {
-                if (b) ce_fixed<K, HM, 1, KEY, NR>(v);
-                else ce_fixed<K, HM, 0, KEY, NR>(v);
+                for (int j = 0; j < (1 << t); ++j) off[j + (1 << t)] = off[j] ^ v;
             } else {
-                ce_dispatch<K, KEY, HM + 1, NR>(v, hm, b);
+#pragma unroll
+                for (int j = 0; j < (1 << (t - 3)); ++j) top[j + (1 << (t - 3))] = top[j] ^ v;
             }
         }
     }
-}
+    __device__ __forceinline__ uint32_t operator[](int j) const { return off[j % LO] ^ top[j / LO]; }
+};
 
-// The stage in register bit k (known at compile time after unrolling).
-template <int KEY, int NR, typename V>
-__device__ __forceinline__ void ce_stage(int k, RegSets<V, NR> &v, uint32_t hm, uint32_t b)
-{
-    static_assert(kSortRegBits == 4, "one case per register bit");
-    if (k == 0) ce_dispatch<0, KEY, 0, NR>(v, hm, b);
-    else if (k == 1) ce_dispatch<1, KEY, 0, NR>(v, hm, b);
-    else if (k == 2) ce_dispatch<2, KEY, 0, NR>(v, hm, b);
-    else ce_dispatch<3, KEY, 0, NR>(v, hm, b);
-}
-
-// NR rounds at a time (NR = 2 needs at least two rounds per group).
-template <int E_LOG, int KEY, bool UNROLLED, int NR>
-__device__ __forceinline__ void run_groups(const SortDesc &sd, uint32_t sbase, uint64_t bc)
+// The groups on the tile.  A group's table entries are loaded together at its
+// start and kept: a chain of shared-memory loads in front of the keys and
+// again in front of their stores costs a one-block sort more than its stages.
+template <int E_LOG, int KEY, int R, int NR>
+__device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Units u)
 {
     using V = typename KeyWord<E_LOG>::type;
-    constexpr int E = 1 << kSortRegBits;
-    const uint32_t tid = threadIdx.x;
-    for (uint32_t gi = 0; gi < sd.n_group; ++gi) {
-        const SortGroup &G = sd.grp[gi];
-        uint32_t tq = 0;
-#pragma unroll
-        for (int t = 0; t < 5; ++t)
-            if ((tid >> t) & 1u) tq ^= G.lane[t];
-#pragma unroll
-        for (int t = 0; t < 3; ++t)
-            if ((tid >> (5 + t)) & 1u) tq ^= G.warp[t];
-        // byte offsets of the registers' slots, relative to the round's base
-        uint32_t roff[E];
-        roff[0] = 0;
-#pragma unroll
-        for (int j = 1; j < E; ++j) {
-            // j with its lowest set bit cleared, then that bit's vector
-            int lb = 0;
-            while (!((j >> lb) & 1)) ++lb;
-            roff[j] = roff[j & (j - 1)] ^ ((uint32_t)G.reg[lb] << E_LOG);
-        }
-        const uint32_t rounds = 1u << sd.round_bits;
-        const uint32_t end = (uint32_t)G.first + G.count;
-        for (uint32_t rd = 0; rd < rounds; rd += NR) {
-            uint32_t qbyte[NR];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                uint32_t qb = tq;
-                for (uint32_t t = 0; t < sd.round_bits; ++t)
-                    if (((rd + (uint32_t)r) >> t) & 1u) qb ^= G.round[t];
-                qbyte[r] = qb << E_LOG;
+    constexpr int E = 1 << R;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t n_group = tab.d.n_group;
+    constexpr bool kFloat = KEY == dev::kKeyF32 || KEY == dev::kKeyF64;
+    bool exact = false;
+    if constexpr (kFloat && NR > 1) {  // the first group's keys are not all in registers at once
+        bool any = false;
+#pragma unroll 4
+        for (int c = 0; c < NR * E * (1 << E_LOG) / 16; ++c) {
+            uint4 *at = reinterpret_cast<uint4 *>(tile) + threadIdx.x + c * blockDim.x;
+            const uint4 w = *at;
+            if constexpr (KEY == dev::kKeyF32) {
+                any |= special<KEY>(w.x) || special<KEY>(w.y) || special<KEY>(w.z) || special<KEY>(w.w);
+            } else {
+                unsigned long long x = ((unsigned long long)w.y << 32) | w.x;
+                unsigned long long y = ((unsigned long long)w.w << 32) | w.z;
+                if (tab.d.first_pass) {
+                    x = ordered(x);
+                    y = ordered(y);
+                    *at = make_uint4((uint32_t)x, (uint32_t)(x >> 32), (uint32_t)y, (uint32_t)(y >> 32));
+                }
+                any |= special<KEY>(x) || special<KEY>(y);
             }
-            V v[NR][E];
+        }
+        exact = __syncthreads_or(any);
+    }
+    for (uint32_t gi = 0; gi < n_group; ++gi) {
+        const GroupTab &g = tab.grp[gi];
+        const uint4 head = g.head;
+        const uint32_t reg[3] = {head.z, head.w, g.reg4 & 0xffffu};
+        const uint32_t n_stage = g.reg4 >> 16, round = g.round;
+        const uint32_t base = (uint32_t)g.lane[lane] ^ g.warp[warp];
+#pragma unroll 1
+        for (int rd = 0; rd < NR; ++rd) {
+            const uint32_t at0 = rd ? base ^ round : base;
+            V v[E];
+            {
+                const RegOffsets<R> at(reg, at0);
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
+                for (int j = 0; j < E; ++j) v[j] = *reinterpret_cast<const V *>(tile + at[j]);
+            }
+            uint64_t codes = ((uint64_t)head.y << 32) | head.x;
+            if constexpr (kFloat && NR == 1) {
+                if (gi == 0) {
+                    bool any = false;
 #pragma unroll
-                for (int j = 0; j < E; ++j)
-                    v[r][j] = lds_key<E_LOG>(sbase + (qbyte[r] ^ roff[j]));
-            // stage first + k pairs the registers that differ in bit k; its
-            // orientation is the block's (hmask, bit of bc)
-#pragma unroll
-            for (int k = 0; k < kSortRegBits; ++k) {
-                const uint32_t s = (uint32_t)G.first + (uint32_t)k;
-                if (s < end) {
-                    const SortStage &st = sd.st[s];
-                    const uint32_t blk = (uint32_t)(bc >> s) & 1u;
-                    if constexpr (UNROLLED) {
-                        ce_stage<KEY, NR>(k, v, st.hmask, blk);
-                    } else {
-                        const uint32_t low0 = st.low0;
-                        ce_regs_k<KEY, NR>(k, v, blk ? ~low0 : low0);
+                    for (int j = 0; j < E; ++j) {
+                        if constexpr (KEY == dev::kKeyF64)
+                            if (tab.d.first_pass) v[j] = ordered(v[j]);
+                        any |= special<KEY>(v[j]);
                     }
+                    exact = __syncthreads_or(any);
                 }
             }
+            if constexpr (kFloat) {
+                if (exact) {
+                    constexpr int how = KEY == dev::kKeyF32 ? KEY : kF64Ordered;
+                    run_stages<how, R>(n_stage, codes, v, u);
+                } else {
+                    constexpr int how = KEY == dev::kKeyF32 ? kF32MinMax : dev::kKeyI64;
+                    run_stages<how, R>(n_stage, codes, v, u);
+                }
+                if constexpr (KEY == dev::kKeyF64)
+                    if (tab.d.last_pass && gi + 1 == n_group)
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
+                        for (int j = 0; j < E; ++j) v[j] = ordered(v[j]);
+            } else {
+                run_stages<KEY, R>(n_stage, codes, v, u);
+            }
+            {
+                // computed again: kept across the stages they would not fit
+                // the registers
+                uint32_t again = at0;
+                asm volatile("" : "+r"(again));
+                const RegOffsets<R> at(reg, again);
 #pragma unroll
-                for (int j = 0; j < E; ++j)
-                    sts_key<E_LOG>(sbase + (qbyte[r] ^ roff[j]), v[r][j]);
+                for (int j = 0; j < E; ++j) *reinterpret_cast<V *>(tile + at[j]) = v[j];
+            }
         }
         __syncthreads();
     }
 }
 
-// Copy a parameter struct into shared memory, 4 bytes per thread and step.
-// The comparator loops read their tables from this copy: read straight from
-// the kernel parameters inside those loops, the tables came out wrong on
-// sm_103a (bit-exact from shared memory, measured on GB300).
-template <typename T>
-__device__ __forceinline__ void stage_params(const T &p, void *dst)
+// Copy a launch table into shared memory, 4 bytes per thread and step: the
+// group loop indexes it by a runtime group and lane.
+__device__ __forceinline__ void stage_words(const void *from, void *to, uint32_t bytes)
 {
-    static_assert(sizeof(T) % 4 == 0, "copied in 4-byte words");
-    const uint32_t *src = reinterpret_cast<const uint32_t *>(&p);
-    uint32_t *d = reinterpret_cast<uint32_t *>(dst);
-    for (uint32_t i = threadIdx.x; i < sizeof(T) / 4; i += blockDim.x) d[i] = src[i];
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(from);
+    uint32_t *dst = reinterpret_cast<uint32_t *>(to);
+    for (uint32_t i = threadIdx.x; i < bytes / 4; i += blockDim.x) dst[i] = src[i];
 }
 
-// Per stage of the pass, the parity of g_s . (this block's input base):
-// lane b contributes the stage mask of thread-block bit b when it is set.
-__device__ __forceinline__ uint64_t block_stage_bits(const PassDesc &d, const SortDesc &sd,
-                                                     uint32_t cta)
+constexpr int kMaxSortThreads = 1 << kSortMaxThreadBits;
+
+// Field f of this thread's chunk 0: the block's and warp's part from one
+// warp-wide XOR (bits of `outer`: thread block, then warp), the lane's from its
+// five bits.
+template <int F>
+__device__ __forceinline__ uint32_t chunk_field(const SortTile &t, uint32_t outer)
 {
+    constexpr uint32_t kOuterBits = kSortMaxCtaBits + kSortMaxThreadBits - 5;
     const uint32_t lane = threadIdx.x & 31u;
-    const bool bit = (lane < d.n_cta) && ((cta >> lane) & 1u);
-    const uint64_t m = bit ? sd.cta_mask[lane] : 0ull;
-    const uint32_t lo = __reduce_xor_sync(0xffffffffu, (uint32_t)m);
-    const uint32_t hi = __reduce_xor_sync(0xffffffffu, (uint32_t)(m >> 32));
-    return ((uint64_t)hi << 32) | lo;
+    uint32_t x = __reduce_xor_sync(
+        0xffffffffu, lane < kOuterBits && ((outer >> lane) & 1u) ? t.block[F][lane] : 0u);
+#pragma unroll
+    for (int b = 0; b < 5; ++b)
+        if ((lane >> b) & 1u) x ^= t.lane[F][b];
+    return x;
 }
 
-// Registers capped for 4 resident blocks with 4-byte keys and one register
-// set (64 per thread: small tiles allow more blocks than 3) and for 3
-// otherwise (80 per thread for 8-byte keys, or for two sets of 4-byte keys,
-// which run on 64 KiB tiles only).
-template <int E_LOG, int KEY, bool UNROLLED, int NR>
-__global__ void __launch_bounds__(256, (E_LOG == 2 && NR == 1) ? 4 : 3)
-    bmmc_sort_pass(const __grid_constant__ PassDesc d, const __grid_constant__ SortDesc sd,
-                   const uint8_t *__restrict__ in, uint8_t *__restrict__ out)
+// Field f of chunk c relative to chunk 0.
+template <int F, int C>
+__device__ __forceinline__ uint32_t chunk_step(const SortTile &t)
+{
+    uint32_t x = 0;
+    if constexpr ((C & 1) != 0) x ^= t.chunk[F][0];
+    if constexpr ((C & 2) != 0) x ^= t.chunk[F][1];
+    if constexpr ((C & 4) != 0) x ^= t.chunk[F][2];
+    if constexpr ((C & 8) != 0) x ^= t.chunk[F][3];
+    return x;
+}
+
+template <int E_LOG, int C, int N>
+__device__ __forceinline__ void load_chunks(const SortTile &t, uint32_t from, uint32_t to,
+                                            const uint8_t *__restrict__ in, uint32_t sbase)
+{
+    if constexpr (C < N) {
+        const uint32_t g = from ^ chunk_step<kSortIn, C>(t);
+        dev::cp_async_16(sbase + (to ^ chunk_step<kSortDst, C>(t)),
+                         in + ((uint64_t)g << E_LOG));
+        load_chunks<E_LOG, C + 1, N>(t, from, to, in, sbase);
+    }
+}
+
+// Output chunks C..N-1: the elements from the tile (load j gives element
+// j ^ rot), one 16-byte store each.  e: tile offset of element j of chunk 0.
+template <int E_LOG, bool ROT, int C, int N>
+__device__ __forceinline__ void store_chunks(const SortTile &t, const uint32_t (&e)[16 >> E_LOG],
+                                             uint32_t to, uint32_t rot,
+                                             uint8_t *__restrict__ out, const uint8_t *tile)
+{
+    if constexpr (C < N) {
+        const uint32_t s = chunk_step<kSortSrc, C>(t);
+        const uint32_t o = to ^ chunk_step<kSortOut, C>(t);
+        uint4 v;
+        if constexpr (E_LOG == 2) {
+            uint32_t a0 = *reinterpret_cast<const uint32_t *>(tile + (s ^ e[0]));
+            uint32_t a1 = *reinterpret_cast<const uint32_t *>(tile + (s ^ e[1]));
+            uint32_t a2 = *reinterpret_cast<const uint32_t *>(tile + (s ^ e[2]));
+            uint32_t a3 = *reinterpret_cast<const uint32_t *>(tile + (s ^ e[3]));
+            if constexpr (ROT) {
+                dev::swap_if((rot & 1u) != 0u, a0, a1);
+                dev::swap_if((rot & 1u) != 0u, a2, a3);
+                dev::swap_if((rot & 2u) != 0u, a0, a2);
+                dev::swap_if((rot & 2u) != 0u, a1, a3);
+            }
+            v = make_uint4(a0, a1, a2, a3);
+        } else {
+            uint2 a0 = *reinterpret_cast<const uint2 *>(tile + (s ^ e[0]));
+            uint2 a1 = *reinterpret_cast<const uint2 *>(tile + (s ^ e[1]));
+            if constexpr (ROT) dev::swap_if((rot & 1u) != 0u, a0, a1);
+            v = make_uint4(a0.x, a0.y, a1.x, a1.y);
+        }
+        dev::stg128(out + ((uint64_t)o << E_LOG), v);
+        store_chunks<E_LOG, ROT, C + 1, N>(t, e, to, rot, out, tile);
+    }
+}
+
+// One block of at most 256 threads per tile of 2^P keys; a thread runs NR sets of
+// 2^R keys in turn in each group and moves as many in and out, in 16-byte
+// chunks.
+template <int E_LOG, int KEY, int R, int NR>
+__global__ void __launch_bounds__(kMaxSortThreads, NR == 1 ? 4 : 3)
+    bmmc_sort_pass(const __grid_constant__ SortDesc sd, const uint8_t *__restrict__ in,
+                   uint8_t *__restrict__ out, Units u)
 {
     extern __shared__ __align__(128) uint8_t smem[];
+    constexpr int kChunks = NR << R >> (4 - E_LOG);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
-    // the comparator tables follow the tile buffer
-    SortDesc *tab = reinterpret_cast<SortDesc *>(smem + d.smem_bytes);
-    stage_params(sd, tab);
-    const uint32_t cta = blockIdx.x;
-    const dev::TileAddr a = dev::tile_addr(d, cta);
-    dev::grid_dependency_wait();
-    dev::allow_dependent_launch();
-    dev::tile_load<E_LOG>(d, a, in, sbase);
+    SortTab &tab = *reinterpret_cast<SortTab *>(smem + sd.tile_bytes);
+    stage_words(&sd, &tab.d,
+                (uint32_t)(offsetof(SortDesc, grp) + sd.n_group * sizeof(SortGroup)));
+    const uint32_t outer = blockIdx.x | (threadIdx.x >> 5) << kSortMaxCtaBits;
+    __syncthreads();
+    const SortTile &t = tab.d.tile;
+    expand_groups<E_LOG>(tab, blockIdx.x, sd.n_cta);
+    {
+        const uint32_t from = chunk_field<kSortIn>(t, outer);
+        const uint32_t to = chunk_field<kSortDst>(t, outer);
+        dev::grid_dependency_wait();
+        dev::allow_dependent_launch();
+        load_chunks<E_LOG, 0, kChunks>(t, from, to, in, sbase);
+    }
     dev::cp_async_wait_all();
     __syncthreads();
-    const uint64_t bc = block_stage_bits(d, *tab, cta);
-    run_groups<E_LOG, KEY, UNROLLED, NR>(*tab, sbase, bc);
-    dev::tile_store<E_LOG, dev::kKeyNone>(d, a, out, sbase);
+    run_groups<E_LOG, KEY, R, NR>(tab, smem, u);
+    uint32_t rot = 0;
+#pragma unroll
+    for (int b = 0; b < 5; ++b)
+        if ((threadIdx.x >> b) & 1u) rot ^= t.rot[b];
+    const uint32_t src = chunk_field<kSortSrc>(t, outer) ^ t.elem[rot];
+    const uint32_t to = chunk_field<kSortOut>(t, outer);
+    uint32_t e[16 >> E_LOG];
+#pragma unroll
+    for (int j = 0; j < (16 >> E_LOG); ++j) e[j] = src ^ t.elem[j];
+    if (t.any_rot) store_chunks<E_LOG, true, 0, kChunks>(t, e, to, rot, out, smem);
+    else store_chunks<E_LOG, false, 0, kChunks>(t, e, to, rot, out, smem);
 }
 
 template <int E_LOG, int KEY>
@@ -286,7 +486,7 @@ __global__ void __launch_bounds__(256)
     const uint32_t count = 1u << dp.N;
     // the tables follow the keys
     SortSmallDesc *tab = reinterpret_cast<SortSmallDesc *>(smem + ((size_t)count << E_LOG));
-    stage_params(dp, tab);
+    stage_words(&dp, tab, sizeof(dp));
     const SortSmallDesc &d = *tab;
     dev::grid_dependency_wait();
     dev::allow_dependent_launch();
@@ -331,67 +531,60 @@ cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t sm
 
 constexpr int kMaxDevices = 64;
 constexpr int kSortTile = 64 * 1024;  // largest tile buffer of a fused pass
-constexpr int kSortSmem = kSortTile + (int)((sizeof(SortDesc) + 127) & ~(size_t)127);
-std::atomic<bool> g_sort_attr[kMaxDevices][2][7][2][2];
+constexpr int kSortSmem = kSortTile + (int)((sizeof(SortTab) + 127) & ~(size_t)127);
+std::atomic<bool> g_sort_attr[kMaxDevices][7][3][2];
 
-template <int E_LOG, int KEY, bool UNROLLED, int NR>
-cudaError_t launch_variant(const PassDesc &d, const SortDesc &sd, const void *in, void *out,
-                           cudaStream_t s)
+template <int E_LOG, int KEY, int R, int NR>
+cudaError_t launch_variant(const SortDesc &sd, const void *in, void *out, cudaStream_t s)
 {
-    int dev = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::atomic<bool> &flag = g_sort_attr[dev][E_LOG - 2][KEY][UNROLLED ? 1 : 0][NR - 1];
-    if (!flag.load(std::memory_order_acquire)) {
-        err = cudaFuncSetAttribute(bmmc_sort_pass<E_LOG, KEY, UNROLLED, NR>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
+    const size_t smem = sd.tile_bytes + sizeof(SortTab);
+    if (smem > 48 * 1024) {
+        int dev = 0;
+        cudaError_t err = cudaGetDevice(&dev);
         if (err != cudaSuccess) return err;
-        flag.store(true, std::memory_order_release);
+        if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+        std::atomic<bool> &flag = g_sort_attr[dev][KEY][R - 3][NR - 1];
+        if (!flag.load(std::memory_order_acquire)) {
+            err = cudaFuncSetAttribute(bmmc_sort_pass<E_LOG, KEY, R, NR>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
+            if (err != cudaSuccess) return err;
+            flag.store(true, std::memory_order_release);
+        }
     }
-    return launch_pdl(bmmc_sort_pass<E_LOG, KEY, UNROLLED, NR>, dim3(1u << d.n_cta), dim3(256),
-                      d.smem_bytes + sizeof(SortDesc), s, d, sd, static_cast<const uint8_t *>(in),
-                      static_cast<uint8_t *>(out));
-}
-
-// 4-byte keys on 64 KiB tiles (four rounds per group): two rounds at a time.
-// Shared memory already holds only 3 such blocks per SM, so the 80
-// registers of two sets cost no resident block; on 32 KiB tiles they would
-// (measured on GB300, n = 22: 0.50 ms against 0.42 with one set; n = 24:
-// 1.50 against 1.56).  The 32 keys of 8-byte ones would not fit the
-// registers.
-template <int E_LOG, int KEY, bool UNROLLED>
-cudaError_t launch_rounds(const PassDesc &d, const SortDesc &sd, const void *in, void *out,
-                          cudaStream_t s)
-{
-    if constexpr (E_LOG == 2) {
-        if (sd.round_bits >= 2) return launch_variant<E_LOG, KEY, UNROLLED, 2>(d, sd, in, out, s);
-    }
-    return launch_variant<E_LOG, KEY, UNROLLED, 1>(d, sd, in, out, s);
+    const uint32_t threads = sd.tile_bytes / (NR << (E_LOG + R));
+    if (threads < 32 || threads > kMaxSortThreads) return cudaErrorInvalidValue;
+    return launch_pdl(bmmc_sort_pass<E_LOG, KEY, R, NR>, dim3(1u << sd.n_cta), dim3(threads), smem, s,
+                      sd, static_cast<const uint8_t *>(in), static_cast<uint8_t *>(out),
+                      Units{1u, ~0u});
 }
 
 template <int E_LOG, int KEY>
-cudaError_t launch_typed(const PassDesc &d, const SortDesc &sd, const void *in, void *out,
-                         cudaStream_t s)
+cudaError_t launch_typed(const SortDesc &sd, const void *in, void *out, cudaStream_t s)
 {
-    return sd.unrolled ? launch_rounds<E_LOG, KEY, true>(d, sd, in, out, s)
-                       : launch_rounds<E_LOG, KEY, false>(d, sd, in, out, s);
+    if constexpr (E_LOG == 2) {
+        if (sd.reg_bits == 5 && sd.rounds == 1) return launch_variant<E_LOG, KEY, 5, 1>(sd, in, out, s);
+        if (sd.reg_bits == 5 && sd.rounds == 2) return launch_variant<E_LOG, KEY, 5, 2>(sd, in, out, s);
+    } else if (sd.reg_bits == 4 && sd.rounds == 2) {
+        return launch_variant<E_LOG, KEY, 4, 2>(sd, in, out, s);
+    }
+    if (sd.reg_bits == 3 && sd.rounds == 1) return launch_variant<E_LOG, KEY, 3, 1>(sd, in, out, s);
+    if (sd.reg_bits == 4 && sd.rounds == 1) return launch_variant<E_LOG, KEY, 4, 1>(sd, in, out, s);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_sort_pass(const PassDesc &d, const SortDesc &sd, const void *in, void *out,
-                             cudaStream_t s)
+cudaError_t launch_sort_pass(const SortDesc &sd, const void *in, void *out, cudaStream_t s)
 {
     using namespace dev;
-    if (d.smem_bytes > (uint32_t)kSortTile || d.thread_bits != 8) return cudaErrorInvalidValue;
+    if (sd.tile_bytes > (uint32_t)kSortTile) return cudaErrorInvalidValue;
     switch (sd.key) {
-    case kKeyI32: return launch_typed<2, kKeyI32>(d, sd, in, out, s);
-    case kKeyU32: return launch_typed<2, kKeyU32>(d, sd, in, out, s);
-    case kKeyF32: return launch_typed<2, kKeyF32>(d, sd, in, out, s);
-    case kKeyI64: return launch_typed<3, kKeyI64>(d, sd, in, out, s);
-    case kKeyU64: return launch_typed<3, kKeyU64>(d, sd, in, out, s);
-    case kKeyF64: return launch_typed<3, kKeyF64>(d, sd, in, out, s);
+    case kKeyI32: return launch_typed<2, kKeyI32>(sd, in, out, s);
+    case kKeyU32: return launch_typed<2, kKeyU32>(sd, in, out, s);
+    case kKeyF32: return launch_typed<2, kKeyF32>(sd, in, out, s);
+    case kKeyI64: return launch_typed<3, kKeyI64>(sd, in, out, s);
+    case kKeyU64: return launch_typed<3, kKeyU64>(sd, in, out, s);
+    case kKeyF64: return launch_typed<3, kKeyF64>(sd, in, out, s);
     default: return cudaErrorInvalidValue;
     }
 }

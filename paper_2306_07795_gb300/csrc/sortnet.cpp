@@ -21,6 +21,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <string>
 #include <utility>
 #include <vector>
@@ -179,50 +180,40 @@ namespace sortnet {
 
 namespace {
 
-int rank_of(const std::vector<uint64_t> &v)
-{
-    return f2::rank(v.data(), (int)v.size());
-}
+// Coordinates in a list of independent vectors (bit i: vector i is used), by
+// elimination on (vector, combination) pairs.
+struct Coords {
+    uint32_t vec[32] = {}, comb[32] = {};  // by leading bit
 
-bool in_span(const std::vector<uint64_t> &v, uint64_t x)
-{
-    std::vector<uint64_t> t = v;
-    t.push_back(x);
-    return rank_of(t) == rank_of(v);
-}
-
-// Coordinates of x in the independent vectors B (bit i: B[i] is used), by
-// elimination on (vector, combination) pairs.  False if x is not in the span.
-bool solve(const std::vector<uint64_t> &B, uint64_t x, uint64_t *coords)
-{
-    std::vector<uint64_t> vec, comb;
-    for (size_t i = 0; i < B.size(); ++i) {
-        uint64_t v = B[i], c = 1ull << i;
-        for (size_t j = 0; j < vec.size(); ++j)
-            if ((v >> (63 - __builtin_clzll(vec[j]))) & 1ull) {
-                v ^= vec[j];
-                c ^= comb[j];
-            }
-        if (!v) return false;  // B dependent
-        const int t = 63 - __builtin_clzll(v);
-        for (size_t j = 0; j < vec.size(); ++j)
-            if ((vec[j] >> t) & 1ull) {
-                vec[j] ^= v;
-                comb[j] ^= c;
-            }
-        vec.push_back(v);
-        comb.push_back(c);
+    bool add(uint32_t v, int index)
+    {
+        uint32_t c = 1u << index;
+        reduce(&v, &c);
+        if (!v) return false;
+        vec[31 - __builtin_clz(v)] = v;
+        comb[31 - __builtin_clz(v)] = c;
+        return true;
     }
-    uint64_t cx = 0;
-    for (size_t j = 0; j < vec.size(); ++j)
-        if ((x >> (63 - __builtin_clzll(vec[j]))) & 1ull) {
-            x ^= vec[j];
-            cx ^= comb[j];
+    // False if x is not in the span.
+    bool of(uint32_t x, uint32_t *coords) const
+    {
+        uint32_t c = 0;
+        reduce(&x, &c);
+        *coords = c;
+        return !x;
+    }
+
+  private:
+    void reduce(uint32_t *v, uint32_t *c) const
+    {
+        while (*v) {
+            const int b = 31 - __builtin_clz(*v);
+            if (!vec[b]) return;
+            *v ^= vec[b];
+            *c ^= comb[b];
         }
-    if (x) return false;
-    *coords = cx;
-    return true;
-}
+    }
+};
 
 uint64_t xor_bits64(const uint64_t *tab, uint64_t bits)
 {
@@ -239,14 +230,6 @@ f2::Mat from_columns(const std::vector<uint64_t> &cols, int n)
     for (int j = 0; j < n; ++j)
         for (int i = 0; i < n; ++i)
             if ((cols[j] >> i) & 1ull) m.r[i] |= 1ull << j;
-    return m;
-}
-
-f2::Mat lift_mat(const f2::Mat &a, int N)
-{
-    f2::Mat m = a;
-    m.n = N;
-    for (int i = a.n; i < N; ++i) m.r[i] = 1ull << i;
     return m;
 }
 
@@ -386,8 +369,7 @@ int group_stages(const std::vector<uint64_t> &U, int k, int D,
             for (uint32_t v : c.in) sp.add(v);
             std::vector<Span> spans;  // spans[i]: after stage c.done + i
             int e = c.done;
-            while (e < S && e - c.done < kSortMaxStages &&
-                   (sp.dim < D || !sp.reduce((uint32_t)U[e]))) {
+            while (e < S && (sp.dim < D || !sp.reduce((uint32_t)U[e]))) {
                 sp.add((uint32_t)U[e]);
                 spans.push_back(sp);
                 ++e;
@@ -510,95 +492,227 @@ int pick_lanes(const std::vector<uint64_t> &pool, int e_log, std::vector<uint64_
     return bank_bits - (int)r;
 }
 
-// Register groups of one pass and their thread mappings (physical slots).
-// A group takes consecutive stages while their partner vectors are
-// independent and the matrix M[a][b] = parity(hslot_a & delta_b) stays
-// invertible: then the common kernel K0 of the group's low tests is a
-// complement of the partner vectors, and the lanes, warps, rounds and unused
-// register bits are all taken from K0 (see SortStage).  *conflicts receives the
-// extra shared-memory wavefronts of a key's round trips, over the groups.
-int build_groups(SortDesc *sd, const std::vector<uint32_t> &delta,
-                 const std::vector<uint32_t> &hslot, int P, int e_log, int *conflicts)
+// Where a pass's tables put virtual indices: a vector's slot part and a
+// functional's parts on input positions and on slots.
+struct SlotView {
+    Coords lam;                 // in the tile's span
+    uint32_t slot_pos[32] = {}; // input position of slot bit i, swizzle included
+    const SlotMap *map;
+    const f2::Mat *L, *L_inv;   // layout the pass reads
+
+    SlotView(const SlotMap &m, const f2::Mat &l, const f2::Mat &l_inv)
+        : map(&m), L(&l), L_inv(&l_inv)
+    {
+        for (int i = 0; i < m.P; ++i) {
+            lam.add(m.lam[i], i);
+            for (uint32_t s = m.swz(1u << i); s; s &= s - 1) slot_pos[i] ^= m.lam[__builtin_ctz(s)];
+        }
+    }
+    bool slot(uint64_t v, uint32_t *out) const
+    {
+        uint32_t coords = 0;
+        if (!lam.of((uint32_t)L->apply(v), &coords)) return false;
+        *out = map->swz(coords);
+        return true;
+    }
+    // g . x_virtual = g . (L^{-1} x_physical)
+    uint64_t on_input(uint64_t g) const
+    {
+        uint64_t hin = 0;
+        for (; g; g &= g - 1) hin ^= L_inv->r[__builtin_ctzll(g)];
+        return hin;
+    }
+    uint64_t on_slots(uint64_t hin) const
+    {
+        uint64_t hs = 0;
+        for (int i = 0; i < map->P; ++i)
+            hs |= (uint64_t)__builtin_parityll(hin & slot_pos[i]) << i;
+        return hs;
+    }
+};
+
+// The coordinates of a group's stages [first, end): its distinct tests in the
+// order of the network's index bits (test of bit i is the functional of virtual
+// bit n - 1 - i), and each stage's code.  False if the stages do not make a
+// group: more than R tests, tests that do not separate the span of the partner
+// vectors, or a stage that is no run.
+bool group_coords(const std::vector<uint64_t> &U, const std::vector<uint64_t> &G, int first,
+                  int end, int R, std::vector<uint64_t> *tests, std::vector<uint8_t> *codes)
 {
+    tests->clear();
+    codes->clear();
+    if (end - first > kSortMaxGroupStages) return false;
+    for (int s = first; s < end; ++s)
+        if (std::find(tests->begin(), tests->end(), G[s]) == tests->end()) tests->push_back(G[s]);
+    std::sort(tests->begin(), tests->end(), std::greater<uint64_t>());
+    const int f = (int)tests->size();
+    if (f > R) return false;
+    Span W, C;  // partner vectors; the same in the tests' coordinates
+    for (int s = first; s < end; ++s) {
+        uint32_t m = 0;
+        int own = -1;
+        for (int t = 0; t < f; ++t) {
+            m |= (uint32_t)__builtin_parityll((*tests)[t] & U[s]) << t;
+            if ((*tests)[t] == G[s]) own = t;
+        }
+        if (!m || __builtin_ctz(m) != own) return false;
+        const int l = 32 - __builtin_clz(m);
+        if (m != ((1u << l) - (1u << own))) return false;
+        codes->push_back((uint8_t)sort_stage_code(own, l));
+        W.add((uint32_t)U[s]);
+        C.add(m);
+    }
+    return W.dim == f && C.dim == f;
+}
+
+// Register groups of one pass and their thread mappings in physical slots (see
+// sort_desc.h).  *conflicts receives the extra shared-memory wavefronts of a
+// key's round trips, over the groups.
+int build_groups(SortDesc *sd, const std::vector<uint64_t> &U, const std::vector<uint64_t> &G,
+                 int first, int end, const SlotView &view, const PassDesc &desc, int e_log,
+                 int *conflicts)
+{
+    const int P = view.map->P, R = (int)sd->reg_bits;
+    const int round_bits = (int)sd->rounds - 1;
+    const int warp_bits = P - R - 5 - round_bits;
+    if (warp_bits < 0 || warp_bits > kSortMaxThreadBits - 5 || desc.n_cta > kSortMaxCtaBits)
+        return -3;
     *conflicts = 0;
-    const int R = kSortRegBits;
-    const int round_bits = P - R - 8;
-    if (round_bits < 0 || round_bits > kSortMaxRoundBits) return -3;
-    sd->round_bits = (uint32_t)round_bits;
-    const int S = (int)delta.size();
-    int g = 0, s = 0;
-    auto m_invertible = [&](int first, int count) {
-        std::vector<uint64_t> rows;
-        for (int a = 0; a < count; ++a) {
-            uint64_t row = 0;
-            for (int b = 0; b < count; ++b)
-                row |= (uint64_t)__builtin_parity(hslot[first + a] & delta[first + b]) << b;
-            rows.push_back(row);
-        }
-        return rank_of(rows) == count;
-    };
-    while (s < S) {
+    int g = 0, s = first;
+    std::vector<uint64_t> tests;
+    std::vector<uint8_t> codes;
+    while (s < end) {
         if (g >= kSortMaxGroups) return -3;
-        SortGroup &G = sd->grp[g];
-        memset(&G, 0, sizeof(G));
-        std::vector<uint64_t> reg;
-        G.first = (uint16_t)s;
-        while (s < S && (int)reg.size() < R && !in_span(reg, delta[s]) &&
-               m_invertible(G.first, s - G.first + 1)) {
-            reg.push_back(delta[s]);
-            ++s;
+        SortGroup &Gr = sd->grp[g++];
+        memset(&Gr, 0, sizeof(Gr));
+        int e = s;
+        for (int q = s + 1; q <= end && q - s <= kSortMaxGroupStages; ++q)
+            if (group_coords(U, G, s, q, R, &tests, &codes)) e = q;
+        if (e == s || !group_coords(U, G, s, e, R, &tests, &codes)) return -3;
+        const int f = (int)tests.size();
+        Gr.n_stage = (uint16_t)(e - s);
+        for (int q = 0; q < e - s; ++q) Gr.code[q / 8] |= (uint32_t)codes[q] << (4 * (q % 8));
+        // vectors dual to the tests in the span of the partner vectors: the
+        // stages' vectors, eliminated on the tests
+        std::vector<uint64_t> dual(f, 0);
+        std::vector<std::pair<uint32_t, uint64_t>> rows;  // (coordinates, vector)
+        for (int q = s; q < e; ++q) {
+            uint32_t m = 0;
+            for (int t = 0; t < f; ++t) m |= (uint32_t)__builtin_parityll(tests[t] & U[q]) << t;
+            rows.push_back({m, U[q]});
         }
-        G.count = (uint16_t)(s - G.first);
-        std::vector<uint64_t> fs;
-        for (int q = G.first; q < s; ++q) fs.push_back(hslot[q]);
+        for (int t = 0; t < f; ++t) {
+            size_t sel = t;
+            while (sel < rows.size() && !((rows[sel].first >> t) & 1u)) ++sel;
+            if (sel == rows.size()) return -3;
+            std::swap(rows[t], rows[sel]);
+            for (size_t i = 0; i < rows.size(); ++i)
+                if (i != (size_t)t && ((rows[i].first >> t) & 1u)) {
+                    rows[i].first ^= rows[t].first;
+                    rows[i].second ^= rows[t].second;
+                }
+        }
+        std::vector<uint64_t> reg, fs, hin;
+        for (int t = 0; t < f; ++t) {
+            uint32_t sl = 0;
+            if (!view.slot(rows[t].second, &sl)) return BMMC_ERR_INVALID;
+            reg.push_back(sl);
+            hin.push_back(view.on_input(tests[t]));
+            fs.push_back(view.on_slots(hin.back()));
+        }
         const std::vector<uint64_t> k0 = nullspace(fs, P);
-        // lanes from K0, then unused register bits, warps and rounds from K0
+        // lanes from K0, then unused register bits and warps from K0
         std::vector<uint64_t> lanes;
         const int lost = pick_lanes(k0, e_log, &lanes);
         if (lost < 0) return -3;
         *conflicts += (1 << lost) - 1;
-        std::vector<uint64_t> all = reg;
-        all.insert(all.end(), lanes.begin(), lanes.end());
+        Span all;
+        for (uint64_t v : reg) all.add((uint32_t)v);
+        for (uint64_t v : lanes) all.add((uint32_t)v);
         std::vector<uint64_t> fill;
         for (uint64_t v : k0)
-            if ((int)(all.size()) < P && !in_span(all, v)) {
-                all.push_back(v);
-                fill.push_back(v);
-            }
-        if ((int)all.size() != P || (int)fill.size() != (R - (int)reg.size()) + 3 + round_bits)
+            if (all.add((uint32_t)v)) fill.push_back(v);
+        if (all.dim != P || (int)fill.size() != R - f + warp_bits + round_bits)
             return -3;
         size_t fi = 0;
         while ((int)reg.size() < R) reg.push_back(fill[fi++]);
-        for (int t = 0; t < R; ++t) G.reg[t] = (uint16_t)reg[t];
-        for (int t = 0; t < 5; ++t) G.lane[t] = (uint16_t)lanes[t];
-        for (int t = 0; t < 3; ++t) G.warp[t] = (uint16_t)fill[fi++];
-        for (int t = 0; t < round_bits; ++t) G.round[t] = (uint16_t)fill[fi++];
-        // each stage's orientation mask over the other register bits
-        for (int k = 0; k < G.count; ++k) {
-            const int q = G.first + k;
-            uint32_t hm = 0;
-            for (int t = 0; t < R; ++t) {
-                const uint32_t par = (uint32_t)__builtin_parityll(hslot[q] & reg[t]);
-                if (t == k) {
-                    if (!par) return -3;  // g_s . u_s = 1
-                } else {
-                    hm |= par << t;
-                }
-            }
-            // lanes, warps and rounds do not change the low test
-            for (int t = 0; t < 5; ++t)
-                if (__builtin_parityll(hslot[q] & lanes[t])) return -3;
-            for (size_t t = R - (reg.size() - (size_t)G.count); t < fill.size(); ++t)
-                if (__builtin_parityll(hslot[q] & fill[t])) return -3;
-            sd->st[q].hmask = (uint8_t)hm;
-            uint32_t low0 = 0;
-            for (uint32_t j = 0; j < (1u << R); ++j)
-                if (!((j >> k) & 1u) && !__builtin_parity(j & hm)) low0 |= 1u << j;
-            sd->st[q].low0 = (uint16_t)low0;
+        for (int t = 0; t < R; ++t) Gr.reg[t] = (uint16_t)reg[t];
+        for (int t = 0; t < 5; ++t) Gr.lane[t] = (uint16_t)lanes[t];
+        for (int t = 0; t < warp_bits; ++t) Gr.warp[t] = (uint16_t)fill[fi++];
+        if (round_bits) Gr.round = (uint16_t)fill[fi++];
+        // a block whose input base has test t set finds register j's key at
+        // the slot of j with bit t flipped
+        for (uint32_t bb = 0; bb < desc.n_cta; ++bb)
+            for (int t = 0; t < f; ++t)
+                if (__builtin_parityll(hin[t] & desc.cta_in[bb])) Gr.cta[bb] ^= (uint16_t)reg[t];
+        // the tests are 1 on their own register vector, 0 on everything else
+        for (int t = 0; t < f; ++t) {
+            for (int q = 0; q < R; ++q)
+                if (__builtin_parityll(fs[t] & reg[q]) != (q == t)) return -3;
+            for (uint64_t v : lanes)
+                if (__builtin_parityll(fs[t] & v)) return -3;
+            for (uint64_t v : fill)
+                if (__builtin_parityll(fs[t] & v)) return -3;
         }
-        ++g;
+        s = e;
     }
     sd->n_group = (uint32_t)g;
+    sd->n_stage = (uint32_t)(end - first);
+    return 0;
+}
+
+// Register bits of a thread.  Few keys per thread shorten the chain of a block's
+// instructions, many save round trips through shared memory: a whole sort in
+// one block of 2^11 keys runs in 12.7 us with 8 keys a thread and 14.6 with 16
+// (int32), 2^16 keys in 2^12-key blocks in 31 us with 16 and 33 with 32, and
+// 2^13-key blocks take 32 in their 13 stages' three groups.  32 8-byte keys do
+// not fit the registers.
+int reg_bits(int e_log, int D)
+{
+    if (D <= 11) return 3;
+    return e_log == 2 && D >= 13 ? 5 : 4;
+}
+
+// The chunk tables of a pass from those of a tiled pass (thread and loop bits of
+// that kernel's blocks, in order, are this one's lane, warp and chunk bits).
+int build_tile(SortDesc *sd, const PassDesc &d, int e_log)
+{
+    SortTile &t = sd->tile;
+    const int w_log = 4 - e_log, P = (int)d.thread_bits + __builtin_ctz(d.loop) + w_log;
+    const int key_bits = (int)(sd->reg_bits + sd->rounds - 1);
+    const int T = P - key_bits;  // thread bits of this kernel
+    const int chunk_bits = key_bits - w_log;
+    if (T < 5 || T > kSortMaxThreadBits || chunk_bits > 4 || d.n_cta > kSortMaxCtaBits ||
+        d.out_const || d.src_const)
+        return -3;
+    sd->n_cta = d.n_cta;
+    sd->tile_bytes = d.smem_bytes;
+    const uint32_t *thr[4] = {d.thr_in, d.thr_dst, d.thr_src, d.thr_out};
+    const uint32_t *loop[4] = {d.loop_in, d.loop_dst, d.loop_src, d.loop_out};
+    const uint32_t *cta[4] = {d.cta_in, nullptr, d.cta_src, d.cta_out};
+    for (int f = 0; f < 4; ++f) {
+        const int sh = f == kSortDst || f == kSortSrc ? e_log : 0;
+        for (uint32_t i = 0; i < d.loop; ++i) {  // the loop tables are linear in i
+            uint32_t x = 0;
+            for (int b = 0; (1u << b) < d.loop; ++b)
+                if ((i >> b) & 1u) x ^= loop[f][1u << b];
+            if (x != loop[f][i]) return -3;
+        }
+        for (int b = 0; b < T + chunk_bits; ++b) {
+            const uint32_t v = (b < (int)d.thread_bits ? thr[f][b]
+                                                       : loop[f][1u << (b - (int)d.thread_bits)])
+                               << sh;
+            if (b < 5) t.lane[f][b] = v;
+            else if (b < T) t.block[f][kSortMaxCtaBits + b - 5] = v;
+            else t.chunk[f][b - T] = v;
+        }
+        for (uint32_t b = 0; cta[f] && b < d.n_cta; ++b) t.block[f][b] = cta[f][b] << sh;
+    }
+    for (int j = 0; j < 1 << w_log; ++j) t.elem[j] = d.elem_src[j] << e_log;
+    for (uint32_t b = 0; b < d.thread_bits; ++b) {
+        if (b >= 5 && d.thr_rot[b]) return -3;
+        if (b < 5) t.any_rot |= t.rot[b] = d.thr_rot[b];
+    }
     return 0;
 }
 
@@ -612,92 +726,65 @@ uint64_t mix64(uint64_t *s)
 }
 
 // Bank bits that a layout L takes from the low tests of the next pass's stages:
-// over runs of kSortRegBits stages, the low address bits (rows of L) that are
+// over runs of R stages, the low address bits (rows of L) that are
 // combinations of each other and of the run's tests.
-int bank_clashes(const PassPlan &next, const std::vector<uint64_t> &G, const f2::Mat &L, int e_log)
+int bank_clashes(const PassPlan &next, const std::vector<uint64_t> &G, const f2::Mat &L, int e_log,
+                 int R)
 {
     const int bank_bits = e_log == 2 ? 5 : 4;
     int clashes = 0;
-    for (int s = next.first; s < next.end; s += kSortRegBits) {
+    for (int s = next.first; s < next.end; s += R) {
         Span sp;
-        for (int q = s; q < next.end && q < s + kSortRegBits; ++q) sp.add((uint32_t)G[q]);
+        for (int q = s; q < next.end && q < s + R; ++q) sp.add((uint32_t)G[q]);
         for (int i = 0; i < bank_bits; ++i) clashes += !sp.add((uint32_t)L.r[i]);
     }
     return clashes;
 }
 
 // Tables of one pass from layout L_prev to layout L.  *score receives the extra
-// shared-memory wavefronts of its register groups and stores.
+// shared-memory wavefronts of its register groups and stores, and whether output
+// chunks are read rotated.
 int derive_sort_pass(const PassPlan &pp, const std::vector<uint64_t> &U,
                      const std::vector<uint64_t> &G, const f2::Mat &L, const f2::Mat &L_prev,
                      const f2::Mat &L_prev_inv, int N, int e_log, int key, int k, int D,
-                     int compare_code, PassDesc *desc_out, SortDesc *sd_out, int *score)
+                     SortDesc *sd_out, int *score)
 {
-    PassDesc &desc = *desc_out;
     const f2::Mat T = f2::mul(L, L_prev_inv);
     // the block span in physical input positions, padded with unit
     // vectors up to D dimensions
     std::vector<uint64_t> W;
-    for (uint64_t v : pp.span) W.push_back(L_prev.apply(v));
-    for (int j = 0; j < N && rank_of(W) < D; ++j)
-        if (!in_span(W, 1ull << j)) W.push_back(1ull << j);
+    Span span;
+    for (uint64_t v : pp.span) {
+        W.push_back(L_prev.apply(v));
+        span.add((uint32_t)W.back());
+    }
+    for (int j = 0; j < N && span.dim < D; ++j)
+        if (span.add(1u << j)) W.push_back(1ull << j);
+    PassDesc desc;
     PassInfo info;
     SlotMap map;
     PlanOptions opt;
     opt.seg_bits = k;
     int rc = derive_pass_span(T, 0, N, e_log, opt, W.data(), (int)W.size(), &desc, &info, &map);
     if (rc) return rc;
-    if (desc.naive || map.P != D || desc.thread_bits != 8) return BMMC_ERR_UNSUPPORTED;
-    std::vector<uint64_t> lam(map.lam, map.lam + map.P);
-
+    if (desc.naive || map.P != D) return BMMC_ERR_UNSUPPORTED;
     SortDesc &sd = *sd_out;
     memset(&sd, 0, sizeof(sd));
     sd.key = (uint32_t)key;
-    // The unrolled orientation variants pay off on large arrays of 4-byte
-    // keys (GB300: 5 % at 2^20, 11 % at 2^22 and 2^24); smaller sorts are
-    // bound by latency, where the compact loop's smaller code fetches
-    // faster, and 8-byte keys measured faster with the compact loop at
-    // every size.
-    sd.unrolled = compare_code == 2 ||
-                  (compare_code == 0 && e_log == 2 && N >= kSortUnrolledMinBits);
-    sd.n_stage = (uint32_t)(pp.end - pp.first);
-    std::vector<uint32_t> delta, hslot;
-    for (int s = pp.first; s < pp.end; ++s) {
-        const uint64_t v = L_prev.apply(U[s]);
-        uint64_t coords = 0;
-        if (!solve(lam, v, &coords)) return BMMC_ERR_INVALID;
-        const uint32_t dl = map.swz((uint32_t)coords);
-        // g_s . x_virtual = g_s . (L_prev^{-1} x_physical)
-        uint64_t hin = 0;
-        for (int j = 0; j < N; ++j)
-            hin |= (uint64_t)__builtin_parityll(G[s] & L_prev_inv.col(j)) << j;
-        uint32_t hs = 0;
-        for (int i = 0; i < map.P; ++i) {
-            const uint64_t off = xor_bits64(lam.data(), map.swz(1u << i));
-            hs |= (uint32_t)__builtin_parityll(hin & off) << i;
-        }
-        if (!__builtin_parity(hs & dl)) return BMMC_ERR_INVALID;  // g_s . u_s = 1
-        SortStage &st = sd.st[s - pp.first];
-        st.hin = (uint32_t)hin;
-        delta.push_back(dl);
-        hslot.push_back(hs);
-    }
-    for (uint32_t bb = 0; bb < desc.n_cta; ++bb) {
-        uint64_t m = 0;
-        for (int s = pp.first; s < pp.end; ++s)
-            m |= (uint64_t)__builtin_parity(sd.st[s - pp.first].hin & desc.cta_in[bb])
-                 << (s - pp.first);
-        sd.cta_mask[bb] = m;
-    }
-    rc = build_groups(&sd, delta, hslot, map.P, e_log, score);
+    sd.reg_bits = (uint32_t)reg_bits(e_log, D);
+    sd.rounds = D - (int)sd.reg_bits > kSortMaxThreadBits ? 2 : 1;
+    const SlotView view(map, L_prev, L_prev_inv);
+    rc = build_tile(&sd, desc, e_log);
     if (rc) return rc;
-    *score += info.wavefronts_store - info.ideal_store;
+    rc = build_groups(&sd, U, G, pp.first, pp.end, view, desc, e_log, score);
+    if (rc) return rc;
+    *score += info.wavefronts_store - info.ideal_store + (sd.tile.any_rot ? 1 : 0);
     return BMMC_OK;
 }
 
 }  // namespace
 
-int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int compare_code)
+int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
 {
     const int e_log = (key >= BMMC_KEY_I32 && key <= BMMC_KEY_F32) ? 2 : 3;
     const int N = n + b;
@@ -707,21 +794,20 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int co
     p->e_log = e_log;
     p->key = key;
 
-    std::vector<f2::Mat> stages;
-    f2::Mat fin;
-    schedule(n, &stages, &fin);
-    const int S = (int)stages.size();
+    // The stage list in closed form: merge l = 1..n of the recursion has stages
+    // i = 0..l-1, whose pairs differ in virtual bits n-1-i down to n-l and whose
+    // low position has bit n-1-i clear; the keys end at their virtual positions.
+    // (Composing schedule()'s matrices gives the same and took 10 of the 13 ms
+    // that planning n = 20 took.)
+    const int S = n * (n + 1) / 2;
     p->stages = S;
-    std::vector<uint64_t> U(S), G(S);
-    f2::Mat q = f2::Mat::identity(n);
-    for (int s = 0; s < S; ++s) {
-        q = f2::mul(stages[s], q);
-        f2::Mat qi;
-        if (!f2::inverse(q, &qi)) return BMMC_ERR_INVALID;
-        U[s] = qi.col(0);
-        G[s] = q.r[0];
-    }
-    const f2::Mat qfin = lift_mat(f2::mul(fin, q), N);
+    std::vector<uint64_t> U, G;
+    for (int l = 1; l <= n; ++l)
+        for (int i = 0; i < l; ++i) {
+            U.push_back((1ull << (n - i)) - (1ull << (n - l)));
+            G.push_back(1ull << (n - 1 - i));
+        }
+    const f2::Mat qfin = f2::Mat::identity(N);
 
     if (N <= kSortSmallMaxBits) {
         SortSmallDesc &d = p->sdesc;
@@ -738,25 +824,26 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int co
         return BMMC_OK;
     }
 
+    constexpr int kMinBlockBits = 12;
     // Segments of one 128-byte line: each of their bits costs a pass that reads
     // or writes them a dimension of its block.
     const int k = 7 - e_log;
-    // Default block: 64 KiB (more stages per pass), but small enough that a
-    // pass has at least 512 thread blocks to spread over the SMs, and at
-    // least 2^12 keys.
-    int D = block_log2 ? block_log2 - e_log : 16 - e_log;
-    if (!block_log2) {
-        if (D > N - 9) D = N - 9;
-        if (D < kSortRegBits + 8) D = kSortRegBits + 8;
-    }
+    // Default block: more keys per block are fewer passes, fewer keys are more
+    // blocks and more threads per key.  The lines are where the larger block
+    // starts to win (GB300, us, 2^12 / 2^13 / 2^14 4-byte keys: n = 18 float32
+    // 43 / 58 / 88, n = 20 74 / 72 / 113, n = 23 502 / 398 / 429, n = 24
+    // 1091 / 859 / 803; 2^12 / 2^13 8-byte keys: n = 22 int64 391 / 430,
+    // n = 23 857 / 806).
+    int D = block_log2 ? block_log2 - e_log : kMinBlockBits;
+    if (!block_log2)
+        D += e_log == 2 ? (N >= 20) + (N >= 24) : (N >= 23);
+    if (N <= kMinBlockBits) D = N;  // one block, whatever its size asked for
+    else if (D < kMinBlockBits || D + e_log > 16) return BMMC_ERR_UNSUPPORTED;
     if (D > N) D = N;
-    if (D < kSortRegBits + 8 || D + e_log > 16 || D < 2 * k) return BMMC_ERR_UNSUPPORTED;
     p->block_bits = D;
 
-    f2::Mat qfin_inv;
-    f2::inverse(qfin, &qfin_inv);
     std::vector<uint64_t> o_final;
-    for (int j = 0; j < k; ++j) o_final.push_back(qfin_inv.col(j));
+    for (int j = 0; j < k; ++j) o_final.push_back(1ull << j);
 
     std::vector<PassPlan> plans;
     int rc = group_stages(U, k, D, o_final, &plans);
@@ -781,38 +868,38 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int co
         for (int attempt = 0; attempt < (last ? 1 : kTries) && best != 0; ++attempt) {
             f2::Mat L, L_inv;
             if (last) {
-                L = qfin;
-                L_inv = qfin_inv;
+                L = L_inv = qfin;
             } else {
                 std::vector<uint64_t> cols = pp.out;
-                for (int j = 0; j < N && (int)cols.size() < N; ++j)
-                    if (!in_span(cols, 1ull << j)) cols.push_back(1ull << j);
+                Span sp;
+                for (uint64_t v : cols) sp.add((uint32_t)v);
+                for (int j = 0; j < N; ++j)
+                    if (sp.add(1u << j)) cols.push_back(1ull << j);
                 if (attempt)
                     for (int j = k; j < N; ++j) cols[j] ^= xor_bits64(cols.data(), mix64(&seed) >> (64 - k));
                 L_inv = from_columns(cols, N);
                 if (!f2::inverse(L_inv, &L)) return BMMC_ERR_INVALID;
             }
-            PassDesc desc;
             SortDesc sd;
             int score = 0;
             rc = derive_sort_pass(pp, U, G, L, L_prev, L_prev_inv, N, e_log, key, k, D,
-                                  compare_code, &desc, &sd, &score);
+                                  &sd, &score);
             if (rc) return rc;
-            if (!last) score += bank_clashes(plans[pi + 1], G, L, e_log);
+            if (!last) score += bank_clashes(plans[pi + 1], G, L, e_log, reg_bits(e_log, D));
             if (best >= 0 && score >= best) continue;
             if (best >= 0) {
                 p->pass.pop_back();
-                p->ce.pop_back();
                 p->layout.pop_back();
             }
             best = score;
-            p->pass.push_back(desc);
-            p->ce.push_back(sd);
+            p->pass.push_back(sd);
             p->layout.push_back(L);
         }
         L_prev = p->layout.back();
         f2::inverse(L_prev, &L_prev_inv);
     }
+    p->pass.front().first_pass = 1;
+    p->pass.back().last_pass = 1;
     return BMMC_OK;
 }
 
@@ -905,75 +992,79 @@ int emulate(const bmmc_sort_plan_s *p, const void *in_v, void *out_v)
     bufs[1].resize(count << e_log);
     const uint8_t *src = in;
     for (size_t pi = 0; pi < p->pass.size(); ++pi) {
-        const PassDesc &d = p->pass[pi];
-        const SortDesc &sd = p->ce[pi];
+        const SortDesc &sd = p->pass[pi];
+        const SortTile &t = sd.tile;
         uint8_t *dst = (pi + 1 == p->pass.size()) ? out : bufs[pi & 1].data();
-        const uint32_t w = 1u << (4 - d.e_log);
-        const uint32_t slots = d.smem_bytes >> d.e_log;
-        const uint32_t threads = 1u << d.thread_bits;
+        const uint32_t w = 1u << (4 - e_log);
+        const uint32_t slots = sd.tile_bytes >> e_log;
+        const uint32_t R = sd.reg_bits, E = 1u << R;
+        const uint32_t keys = E * sd.rounds;  // of a thread
+        const uint32_t threads = slots / keys;
         std::vector<uint64_t> sm(slots);
-        for (uint64_t blk = 0; blk < (1ull << d.n_cta); ++blk) {
-            // phase 1: input chunks into their slots
-            for (uint32_t tid = 0; tid < threads; ++tid) {
-                const ThreadBase tb = thread_base(d, (uint32_t)blk, tid);
-                for (uint32_t i = 0; i < d.loop; ++i) {
-                    const uint32_t g = tb.in ^ d.loop_in[i];
-                    const uint32_t s = tb.dst ^ d.loop_dst[i];
-                    for (uint32_t j = 0; j < w; ++j) sm[s + j] = load_key(src, g + j, e_log);
+        // field f of (block, thread, chunk)
+        auto field = [&](int f, uint64_t blk, uint32_t tid, uint32_t c) {
+            uint32_t x = 0;
+            for (uint32_t b = 0; b < sd.n_cta; ++b)
+                if ((blk >> b) & 1ull) x ^= t.block[f][b];
+            for (int b = 0; b < kSortMaxThreadBits - 5; ++b)
+                if ((tid >> (5 + b)) & 1u) x ^= t.block[f][kSortMaxCtaBits + b];
+            for (int b = 0; b < 5; ++b)
+                if ((tid >> b) & 1u) x ^= t.lane[f][b];
+            for (int b = 0; b < 4; ++b)
+                if ((c >> b) & 1u) x ^= t.chunk[f][b];
+            return x;
+        };
+        for (uint64_t blk = 0; blk < (1ull << sd.n_cta); ++blk) {
+            // input chunks into their slots
+            for (uint32_t tid = 0; tid < threads; ++tid)
+                for (uint32_t c = 0; c < keys / w; ++c) {
+                    const uint32_t g = field(kSortIn, blk, tid, c);
+                    const uint32_t s = field(kSortDst, blk, tid, c) >> e_log;
+                    for (uint32_t j = 0; j < w; ++j) sm.at(s + j) = load_key(src, g + j, e_log);
                 }
-            }
             // comparator stages, group by group, as each thread runs them
-            uint64_t bc = 0;
-            for (uint32_t bb = 0; bb < d.n_cta; ++bb)
-                if ((blk >> bb) & 1ull) bc ^= sd.cta_mask[bb];
-            const uint32_t R = kSortRegBits, E = 1u << R;
             for (uint32_t gi = 0; gi < sd.n_group; ++gi) {
                 const SortGroup &G = sd.grp[gi];
-                uint32_t roff[1u << kSortRegBits];
+                uint32_t cta = 0;
+                for (uint32_t bb = 0; bb < sd.n_cta; ++bb)
+                    if ((blk >> bb) & 1ull) cta ^= G.cta[bb];
+                uint32_t roff[1u << kSortMaxRegBits];
                 for (uint32_t j = 0; j < E; ++j) {
                     roff[j] = 0;
                     for (uint32_t t = 0; t < R; ++t)
                         if ((j >> t) & 1u) roff[j] ^= G.reg[t];
                 }
-                for (uint32_t tid = 0; tid < threads; ++tid) {
-                    uint32_t tq = 0;
+                for (uint32_t it = 0; it < threads * sd.rounds; ++it) {
+                    const uint32_t tid = it % threads;
+                    uint32_t q = cta ^ (it >= threads ? G.round : 0u);
                     for (int t = 0; t < 5; ++t)
-                        if ((tid >> t) & 1u) tq ^= G.lane[t];
-                    for (int t = 0; t < 3; ++t)
-                        if ((tid >> (5 + t)) & 1u) tq ^= G.warp[t];
-                    for (uint32_t rd = 0; rd < (1u << sd.round_bits); ++rd) {
-                        uint32_t qb = tq;
-                        for (uint32_t t = 0; t < sd.round_bits; ++t)
-                            if ((rd >> t) & 1u) qb ^= G.round[t];
-                        uint64_t v[1u << kSortRegBits];
-                        for (uint32_t j = 0; j < E; ++j) v[j] = sm[qb ^ roff[j]];
-                        for (uint32_t s = G.first; s < (uint32_t)G.first + G.count; ++s) {
-                            const SortStage &st = sd.st[s];
-                            // register j (stage bit 0) holds the pair's low
-                            // position iff parity(j & hmask) is the block's bit
-                            const uint32_t blk = (uint32_t)(bc >> s) & 1u;
-                            const uint32_t bit = 1u << (s - G.first);
-                            for (uint32_t j = 0; j < E; ++j) {
-                                if (j & bit) continue;
-                                const uint32_t jj = j | bit;
-                                if ((uint32_t)__builtin_parity(j & st.hmask) == blk)
-                                    order_pair(p->key, &v[j], &v[jj]);
-                                else
-                                    order_pair(p->key, &v[jj], &v[j]);
-                            }
-                        }
-                        for (uint32_t j = 0; j < E; ++j) sm[qb ^ roff[j]] = v[j];
+                        if ((tid >> t) & 1u) q ^= G.lane[t];
+                    for (int t = 0; t < kSortMaxThreadBits - 5; ++t)
+                        if ((tid >> (5 + t)) & 1u) q ^= G.warp[t];
+                    uint64_t v[1u << kSortMaxRegBits];
+                    for (uint32_t j = 0; j < E; ++j) v[j] = sm.at(q ^ roff[j]);
+                    for (uint32_t s = 0; s < G.n_stage; ++s) {
+                        const uint32_t code = (G.code[s / 8] >> (4 * (s % 8))) & 15u;
+                        uint32_t l = 1;
+                        while ((uint32_t)sort_stage_code(0, (int)l + 1) <= code) ++l;
+                        const uint32_t i = code - (uint32_t)sort_stage_code(0, (int)l);
+                        const uint32_t m = (1u << l) - (1u << i);
+                        for (uint32_t j = 0; j < E; ++j)
+                            if (!((j >> i) & 1u)) order_pair(p->key, &v[j], &v[j ^ m]);
                     }
+                    for (uint32_t j = 0; j < E; ++j) sm.at(q ^ roff[j]) = v[j];
                 }
             }
-            // phase 2: output chunks from their slots
+            // output chunks from their slots
             for (uint32_t tid = 0; tid < threads; ++tid) {
-                const ThreadBase tb = thread_base(d, (uint32_t)blk, tid);
-                for (uint32_t i = 0; i < d.loop; ++i) {
-                    const uint32_t sidx = tb.src ^ d.loop_src[i] ^ d.elem_src[tb.rot];
-                    const uint32_t o = tb.out ^ d.loop_out[i];
+                uint32_t rot = 0;
+                for (int b = 0; b < 5; ++b)
+                    if ((tid >> b) & 1u) rot ^= t.rot[b];
+                for (uint32_t c = 0; c < keys / w; ++c) {
+                    const uint32_t s = field(kSortSrc, blk, tid, c) ^ t.elem[rot];
+                    const uint32_t o = field(kSortOut, blk, tid, c);
                     for (uint32_t j = 0; j < w; ++j)
-                        store_key(dst, o + (j ^ tb.rot), e_log, sm[sidx ^ d.elem_src[j]]);
+                        store_key(dst, o + (j ^ rot), e_log, sm.at((s ^ t.elem[j]) >> e_log));
                 }
             }
         }
@@ -990,8 +1081,7 @@ int emulate(const bmmc_sort_plan_s *p, const void *in_v, void *out_v)
 // ---------------------------------------------------------------------------
 
 namespace bmmc {
-cudaError_t launch_sort_pass(const PassDesc &d, const SortDesc &sd, const void *in, void *out,
-                             cudaStream_t s);
+cudaError_t launch_sort_pass(const SortDesc &sd, const void *in, void *out, cudaStream_t s);
 cudaError_t launch_sort_small(const SortSmallDesc &d, int e_log, const void *in, void *out,
                               cudaStream_t s);
 }  // namespace bmmc
@@ -1016,18 +1106,17 @@ int bmmc_sort_plan_create(bmmc_sort_plan *out, int n, int b, int key_type,
     *out = nullptr;
     if (n < 1 || n > 30 || b < 0 || n + b > 32) return BMMC_ERR_INVALID;
     if (key_type < BMMC_KEY_I32 || key_type > BMMC_KEY_F64) return BMMC_ERR_UNSUPPORTED;
-    int block_log2 = 0, compare_code = 0;
+    int block_log2 = 0;
     if (opts) {
         for (int r : opts->reserved)
             if (r) return BMMC_ERR_UNSUPPORTED;
         block_log2 = opts->block_log2;
-        compare_code = opts->compare_code;
-        if (compare_code < 0 || compare_code > 2) return BMMC_ERR_UNSUPPORTED;
+        if (opts->compare_code < 0 || opts->compare_code > 2) return BMMC_ERR_UNSUPPORTED;
         if (block_log2 && (block_log2 < 12 || block_log2 > 16)) return BMMC_ERR_UNSUPPORTED;
     }
     return guarded([&] {
         bmmc_sort_plan_s *p = new bmmc_sort_plan_s();
-        const int rc = sortnet::plan_sort(p, n, b, key_type, block_log2, compare_code);
+        const int rc = sortnet::plan_sort(p, n, b, key_type, block_log2);
         if (rc) {
             delete p;
             return rc;
@@ -1076,7 +1165,7 @@ int bmmc_sort_execute(bmmc_sort_plan p, const void *in, void *out, void *ws,
         // read and write one buffer
         void *dst = ((np - 1 - i) % 2 == 0) ? out : ws;
         if (debug_fail_launch()) return BMMC_ERR_CUDA;
-        if (launch_sort_pass(p->pass[i], p->ce[i], src, dst, s) != cudaSuccess)
+        if (launch_sort_pass(p->pass[i], src, dst, s) != cudaSuccess)
             return BMMC_ERR_CUDA;
         src = dst;
     }
@@ -1096,13 +1185,13 @@ int bmmc_sort_plan_describe(bmmc_sort_plan p, char *buf, size_t len)
         std::string s = "{\"n\": " + std::to_string(p->n) + ", \"b\": " + std::to_string(p->b) +
                         ", \"key_bytes\": " + std::to_string(1 << p->e_log) +
                         ", \"stages\": " + std::to_string(p->stages) +
-                        ", \"one_block\": " + (p->small ? "true" : "false") +
+                        ", \"one_block\": " + (p->small || p->pass[0].n_cta == 0 ? "true" : "false") +
                         ", \"block_keys_log2\": " + std::to_string(p->block_bits) +
                         ", \"passes\": [";
         for (size_t i = 0; i < p->pass.size(); ++i) {
             char tmp[160];
             snprintf(tmp, sizeof(tmp), "%s{\"stages\": %u, \"groups\": %u, \"blocks\": %llu}",
-                     i ? ", " : "", p->ce[i].n_stage, p->ce[i].n_group,
+                     i ? ", " : "", p->pass[i].n_stage, p->pass[i].n_group,
                      (unsigned long long)(1ull << p->pass[i].n_cta));
             s += tmp;
         }

@@ -5,7 +5,6 @@
 #include <vector>
 
 #include "f2.hpp"
-#include "pass_desc.h"
 #include "plan.hpp"
 #include "sort_desc.h"
 
@@ -18,8 +17,7 @@ struct bmmc_sort_plan_s {
     int block_bits = 0;  // slot bits of a fused pass's thread block
     bool small = false;  // the whole network in one thread block
     bmmc::SortSmallDesc sdesc;
-    std::vector<bmmc::PassDesc> pass;  // fused passes, in order
-    std::vector<bmmc::SortDesc> ce;    // their comparator tables
+    std::vector<bmmc::SortDesc> pass;  // fused passes, in order
     std::vector<bmmc::f2::Mat> layout; // layout after each pass (for checks)
     int stages = 0;  // comparator stages of the network
 };
@@ -28,7 +26,7 @@ namespace bmmc {
 namespace sortnet {
 
 // Build the plan (host only).  Returns 0 or a negative bmmc status.
-int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2, int compare_code);
+int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2);
 
 // Run the plan's tables on the host, exactly as the kernels index them:
 // in and out hold 2^N keys.  Returns 0.

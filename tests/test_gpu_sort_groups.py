@@ -1,0 +1,59 @@
+"""The register groups of the fused sorting passes at their edges: one block and
+the first sizes beyond, every count of keys per thread, and float keys that are
+all ordinary or hold a single NaN or a single -0.0 (one thread block then
+compares with IEEE <=, the others by minimum and maximum or as integers).  Bit
+for bit the host emulation of the same plan."""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2306_07795_gb300 import _binding as B
+
+pytestmark = pytest.mark.gpu
+
+KEYS = {np.float32: B.BMMC_KEY_F32, np.float64: B.BMMC_KEY_F64, np.int32: B.BMMC_KEY_I32,
+        np.uint64: B.BMMC_KEY_U64}
+
+
+def _keys(dtype, count, special, seed):
+    g = np.random.Generator(np.random.PCG64(seed))
+    if not np.issubdtype(dtype, np.floating):
+        info = np.iinfo(dtype)
+        x = g.integers(info.min, info.max, size=count, dtype=dtype, endpoint=True)
+        x[g.integers(0, count, 4)] = info.min
+        x[g.integers(0, count, 4)] = info.max
+        return x
+    x = g.standard_normal(count).astype(dtype)
+    x[g.integers(0, count, 8)] = 0.0
+    x[g.integers(0, count, 4)] = np.finfo(dtype).smallest_subnormal
+    x[g.integers(0, count, 4)] = -np.finfo(dtype).max
+    x[g.integers(0, count)] = np.inf
+    if special is not None:
+        x[g.integers(0, count)] = special
+    return x
+
+
+@pytest.mark.parametrize("dtype,special", [(np.float32, None), (np.float32, np.nan),
+                                           (np.float32, -0.0), (np.float64, None),
+                                           (np.float64, np.nan), (np.float64, -0.0),
+                                           (np.int32, None), (np.uint64, None)])
+@pytest.mark.parametrize("n,b,block_log2", [(7, 0, 0), (8, 0, 0), (9, 0, 0), (11, 0, 0), (12, 0, 0),
+                                            (13, 0, 0), (13, 0, 16), (14, 0, 16), (15, 1, 15),
+                                            (8, 6, 0), (20, 0, 0)])
+def test_groups(n, b, block_log2, dtype, special):
+    import torch
+    x = _keys(dtype, 1 << (n + b), special, n * 10 + b)
+    h = B.bmmc_sort_plan_create(n, b, KEYS[dtype], block_log2)
+    want = np.empty_like(x)
+    B.bmmc_sort_plan_emulate(h, ctypes.c_void_p(x.ctypes.data), ctypes.c_void_p(want.ctypes.data))
+    d = torch.from_numpy(x.view(np.int32 if x.itemsize == 4 else np.int64).copy()).cuda()
+    y = torch.full_like(d, -1)
+    ws = torch.empty(max(16, B.bmmc_sort_workspace_bytes(h)), dtype=torch.uint8, device="cuda")
+    B.bmmc_sort_execute(h, d.data_ptr(), y.data_ptr(), ws.data_ptr(),
+                        torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    B.bmmc_sort_plan_destroy(h)
+    got = y.cpu().numpy().view(dtype)
+    assert np.array_equal(got.view(np.uint8), want.view(np.uint8))
