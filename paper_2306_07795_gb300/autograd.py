@@ -41,15 +41,16 @@ def _apply(plan, x):
         raise ValueError("last dimension holds %d bytes, the plan needs %d"
                          % (last, plan.nbytes))
     rows_total = x.numel() // x.shape[-1]
-    lifted = _lifted_plan(plan, rows_total) if rows_total > 1 else plan
-    if lifted is not None:
-        return lifted(x.view(-1)).view(x.shape)
     # an odd count of groups of 2^b rows, each group one array of the lifted plan
-    b = min((rows_total & -rows_total).bit_length() - 1, 32 - plan.n)
-    out = _lifted_plan(plan, 1 << b).run_rows(x, rows_total >> b)
+    b = min((rows_total & -rows_total).bit_length() - 1, 32 - plan.n) if rows_total > 1 else 0
+    lifted = _lifted_plan(plan, 1 << b) if b else plan
+    groups = max(rows_total >> b, 1)
+    out = lifted.run_rows(x, groups)
     if out is not None:
         return out
-    out = torch.empty_like(x)  # a plan of two launches: row by row
+    if groups == 1:  # plans of two launches
+        return lifted(x.view(-1)).view(x.shape)
+    out = torch.empty_like(x)
     xf, of = x.view(rows_total, -1), out.view(rows_total, -1)
     for r in range(rows_total):
         plan(xf[r], out=of[r])

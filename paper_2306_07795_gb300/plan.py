@@ -7,14 +7,27 @@ two tiled passes (Sec. 4), all done on the host by the C library."""
 from . import _binding as B
 
 
-def _current_raw_stream(dev):
-    """The cudaStream_t of PyTorch's current stream on `dev`, as an int.  The
-    raw accessor skips building a Stream object (about 3 us per call)."""
+_raw_stream_getter = None
+
+
+def current_raw_stream(index):
+    """The cudaStream_t of PyTorch's current stream on CUDA device `index`, as an
+    int.  The raw accessor skips building a Stream object (2 us of a call)."""
+    global _raw_stream_getter
+    if _raw_stream_getter is None:
+        import torch
+        _raw_stream_getter = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+            lambda i: torch.cuda.current_stream(i).cuda_stream)
+    return _raw_stream_getter(index)
+
+
+def on_device(index, fn, *args):
+    """fn(*args) with CUDA device `index` current; returns its result."""
     import torch
-    getter = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if getter is not None:
-        return getter(dev.index)
-    return torch.cuda.current_stream(dev).cuda_stream
+    if index == torch.cuda.current_device():
+        return fn(*args)
+    with torch.cuda.device(index):
+        return fn(*args)
 
 
 class Plan:
@@ -43,7 +56,10 @@ class Plan:
                                             cta_tile_log2, tile_order)
         self._inverse = None
         self._ws_bytes = None
-        self._direct = B.bmmc_plan_num_launches(self._h) == 1
+        self._nbytes = (1 << self.n) * self.elem_bytes
+        # plans are immutable: what a call needs of the library, looked up once
+        self._direct = (B.lib().bmmc_execute_direct
+                        if B.bmmc_plan_num_launches(self._h) == 1 else None)
 
     # -- plan queries -------------------------------------------------------
     @property
@@ -52,7 +68,7 @@ class Plan:
 
     @property
     def nbytes(self):
-        return (1 << self.n) * self.elem_bytes
+        return self._nbytes
 
     @property
     def num_passes(self):
@@ -103,9 +119,9 @@ class Plan:
             raise ValueError("%s must be a CUDA tensor (there is no CPU path)" % name)
         if not t.is_contiguous():
             raise ValueError("%s must be contiguous" % name)
-        if t.numel() * t.element_size() != self.nbytes:
+        if t.numel() * t.element_size() != self._nbytes:
             raise ValueError("%s holds %d bytes, the plan needs %d"
-                             % (name, t.numel() * t.element_size(), self.nbytes))
+                             % (name, t.numel() * t.element_size(), self._nbytes))
 
     def __call__(self, x, out=None, stream=None, workspace=None):
         """Permute tensor x (any dtype; its bytes are 2^n elements of
@@ -117,51 +133,41 @@ class Plan:
             out = torch.empty_like(x)
         else:
             self._check_tensor(out, "out")
-        dev = x.device
-        raw = stream.cuda_stream if stream is not None else _current_raw_stream(dev)
-        if workspace is None and self._direct:
-            def run():
-                return B.lib().bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), 1, raw)
+        dev = x.get_device()
+        raw = stream.cuda_stream if stream is not None else current_raw_stream(dev)
+        if workspace is None and self._direct is not None:
+            code = on_device(dev, self._direct, self._h, x.data_ptr(), out.data_ptr(), 1, raw)
         else:
             ws_bytes = self._ws_bytes
             if ws_bytes is None:
-                ws_bytes = self._ws_bytes = self.workspace_bytes  # plans are immutable
+                ws_bytes = self._ws_bytes = self.workspace_bytes
             if ws_bytes and workspace is None:
-                workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
+                workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=x.device)
             ws_ptr = workspace.data_ptr() if ws_bytes else None
-
-            def run():
-                return B.lib().bmmc_execute_ws(self._h, x.data_ptr(), out.data_ptr(), ws_ptr,
-                                               raw)
-        if dev.index == torch.cuda.current_device():
-            code = run()
-        else:
-            with torch.cuda.device(dev):
-                code = run()
+            code = on_device(dev, B.lib().bmmc_execute_ws, self._h, x.data_ptr(),
+                             out.data_ptr(), ws_ptr, raw)
         if code != B.BMMC_OK:
             raise B.BmmcError(code, "bmmc_execute_ws")
         return out
 
     def run_rows(self, x, rows):
         """Permute each of the `rows` arrays of the contiguous CUDA tensor x
-        alike, in one launch (bmmc_execute_direct).  Returns a new tensor, or
-        None for a plan of two launches."""
+        alike, in one launch (bmmc_execute_direct).  Returns a new contiguous
+        tensor of x's shape, or None for a plan of two launches."""
         import torch
 
-        if not self._direct:
+        if self._direct is None:
             return None
         if not (x.is_cuda and x.is_contiguous()
-                and x.numel() * x.element_size() == rows * self.nbytes):
+                and x.numel() * x.element_size() == rows * self._nbytes):
             raise ValueError("x must be a contiguous CUDA tensor of %d bytes"
-                             % (rows * self.nbytes))
-        out = torch.empty_like(x)
-        dev = x.device
-        raw = _current_raw_stream(dev)
-        if dev.index == torch.cuda.current_device():
-            B.bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), rows, raw)
-        else:
-            with torch.cuda.device(dev):
-                B.bmmc_execute_direct(self._h, x.data_ptr(), out.data_ptr(), rows, raw)
+                             % (rows * self._nbytes))
+        out = torch.empty_like(x, memory_format=torch.contiguous_format)
+        dev = x.get_device()
+        code = on_device(dev, self._direct, self._h, x.data_ptr(), out.data_ptr(), rows,
+                         current_raw_stream(dev))
+        if code != B.BMMC_OK:
+            raise B.BmmcError(code, "bmmc_execute_direct")
         return out
 
     def execute_host(self, host_in, host_out, dev_in, dev_out, stream=None, workspace=None):

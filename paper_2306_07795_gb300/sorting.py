@@ -26,7 +26,7 @@ plans from bmmc_plan_lift; the data path is entirely library kernels.
 """
 
 from . import _binding as B
-from .plan import Plan
+from .plan import Plan, current_raw_stream, on_device
 
 _KEYS = {}
 
@@ -153,19 +153,19 @@ class SortingNetwork:
         b = rows_total.bit_length() - 1
         if rows_total != 1 << b:
             raise ValueError("leading dimensions must hold a power-of-two count of rows")
-        if stream is None:
-            stream = torch.cuda.current_stream(x.device)
         src = x.contiguous()
         if self.fused:
             sp = self._sort_plan(key, b)
             out = torch.empty_like(src)
             ws = torch.empty(sp.ws_bytes, dtype=torch.uint8, device=x.device) \
                 if sp.ws_bytes else None
-            with torch.cuda.device(x.device):
-                B.bmmc_sort_execute(sp.h, src.data_ptr(), out.data_ptr(),
-                                    ws.data_ptr() if ws is not None else None,
-                                    stream.cuda_stream)
+            dev = x.get_device()
+            on_device(dev, B.bmmc_sort_execute, sp.h, src.data_ptr(), out.data_ptr(),
+                      ws.data_ptr() if ws is not None else None,
+                      stream.cuda_stream if stream is not None else current_raw_stream(dev))
             return out
+        if stream is None:
+            stream = torch.cuda.current_stream(x.device)
         stages, final = self._plans_for(elem_bytes, b)
         bufs = [torch.empty_like(src), torch.empty_like(src)]
         cur = src
