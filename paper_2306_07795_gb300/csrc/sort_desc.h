@@ -47,8 +47,16 @@ constexpr int kSortSmallMaxStages = 28;  // 7 * 8 / 2
 // The stage pairing register j with j ^ (ones at bits i..l-1), bit i low.
 constexpr BMMC_HD int sort_stage_code(int i, int l) { return l * (l - 1) / 2 + i; }
 
+// A group of f stages that are the f exchanges (i, f) of its tests in cyclic order
+// from i = r, as whole groups of a merge are (r = 0, or r > 0 where the group
+// runs over the end of a merge into the next).
+constexpr BMMC_HD int sort_cycle_kind(int f, int r) { return f * (f - 1) / 2 + r + 1; }
+// The group that is the first R merges of the network.
+constexpr int kSortLevelsKind = sort_cycle_kind(kSortMaxRegBits, kSortMaxRegBits - 1) + 1;
+
 struct SortGroup {
-    uint16_t n_stage;                // stages of the group
+    uint8_t n_stage;                 // stages of the group
+    uint8_t kind;                    // sort_cycle_kind, kSortLevelsKind, or 0 for any other
     uint16_t reg[kSortMaxRegBits];   // slot vector of register bit t
     uint32_t code[2];                // sort_stage_code of stage s: 4 bits at 4 s
     uint16_t lane[5];                // slot vector of lane bit t

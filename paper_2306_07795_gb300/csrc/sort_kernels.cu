@@ -103,9 +103,10 @@ __device__ __forceinline__ unsigned long long other(unsigned long long a, unsign
 
 // How many pairs of four take their other key from multiply-adds: the compares,
 // minima and selects of a pair run on the ALU pipe at half the issue rate, and
-// sharing the work with the multiply-add pipe is faster.  n = 24, none / two /
-// three / all of four, us: int32 769 / 742 / 747 / 753, float32 830 / 801 / 811 /
-// 811, int64 1991 / 1814 / 1717 / 1673, float64 2198 / 2008 / 1926 / 1913.
+// sharing the work with the multiply-add pipe is faster.  n = 24, none / one /
+// two / three / all of four, us: int32 702 / 696 / 685 / 675 / 695, float32
+// 768 / 738 / 717 / 731 / 755 (the smaller sorts are fastest with two); int64
+// 1916 / 1840 / - / 1656 / 1577, float64 2120 / 2042 / - / 1833 / 1762.
 template <typename V> constexpr int kMadPairs = sizeof(V) == 4 ? 2 : 4;
 
 // Order the pair: a becomes the low one, b the high one.
@@ -173,7 +174,54 @@ __device__ __forceinline__ void ce_stage(uint32_t code, V (&v)[1 << R], Units u)
     }
 }
 
-// The stages of a group.
+// The stages of a group of kind sort_cycle_kind(F, FIRST).
+template <int HOW, int R, int F, int FIRST, int S = 0, typename V>
+__device__ __forceinline__ void run_cycle(V (&v)[1 << R], Units u)
+{
+    if constexpr (F <= R && S < F) {
+        ce_run<(FIRST + S) % F, F, HOW, R>(v, u);
+        run_cycle<HOW, R, F, FIRST, S + 1>(v, u);
+    }
+}
+
+// The first R merges, from stage I of merge L.
+template <int HOW, int R, int L = 1, int I = 0, typename V>
+__device__ __forceinline__ void run_levels(V (&v)[1 << R], Units u)
+{
+    if constexpr (L <= R) {
+        ce_run<I, L, HOW, R>(v, u);
+        if constexpr (I + 1 < L) run_levels<HOW, R, L, I + 1>(v, u);
+        else run_levels<HOW, R, L + 1, 0>(v, u);
+    }
+}
+
+// The stages of a group whose kind is not 0: no choice between stages, which for
+// a few warps costs more than the exchanges do (against run_stages alone, int32:
+// n = 11 9.8 -> 7.2 us, n = 16 28.2 -> 22.6, n = 24 739 -> 685).
+template <int HOW, int R, typename V>
+__device__ __forceinline__ void run_kind(uint32_t kind, V (&v)[1 << R], Units u)
+{
+    switch (kind) {
+    case sort_cycle_kind(1, 0): run_cycle<HOW, R, 1, 0>(v, u); break;
+    case sort_cycle_kind(2, 0): run_cycle<HOW, R, 2, 0>(v, u); break;
+    case sort_cycle_kind(2, 1): run_cycle<HOW, R, 2, 1>(v, u); break;
+    case sort_cycle_kind(3, 0): run_cycle<HOW, R, 3, 0>(v, u); break;
+    case sort_cycle_kind(3, 1): run_cycle<HOW, R, 3, 1>(v, u); break;
+    case sort_cycle_kind(3, 2): run_cycle<HOW, R, 3, 2>(v, u); break;
+    case sort_cycle_kind(4, 0): run_cycle<HOW, R, 4, 0>(v, u); break;
+    case sort_cycle_kind(4, 1): run_cycle<HOW, R, 4, 1>(v, u); break;
+    case sort_cycle_kind(4, 2): run_cycle<HOW, R, 4, 2>(v, u); break;
+    case sort_cycle_kind(4, 3): run_cycle<HOW, R, 4, 3>(v, u); break;
+    case sort_cycle_kind(5, 0): run_cycle<HOW, R, 5, 0>(v, u); break;
+    case sort_cycle_kind(5, 1): run_cycle<HOW, R, 5, 1>(v, u); break;
+    case sort_cycle_kind(5, 2): run_cycle<HOW, R, 5, 2>(v, u); break;
+    case sort_cycle_kind(5, 3): run_cycle<HOW, R, 5, 3>(v, u); break;
+    case sort_cycle_kind(5, 4): run_cycle<HOW, R, 5, 4>(v, u); break;
+    case kSortLevelsKind: run_levels<HOW, R>(v, u); break;
+    }
+}
+
+// The stages of a group, one by one.
 template <int HOW, int R, typename V>
 __device__ __forceinline__ void run_stages(uint32_t n_stage, uint64_t codes, V (&v)[1 << R], Units u)
 {
@@ -197,7 +245,7 @@ __device__ __forceinline__ uint32_t xor_table(const uint16_t *tab, uint32_t v)
 // a few words, offsets of its lanes (the block's own part included) and warps.
 struct GroupTab {
     uint4 head;      // codes; register offsets 0 | 1 << 16, 2 | 3 << 16
-    uint32_t reg4;   // register offset 4 | stages << 16
+    uint32_t reg4;   // register offset 4 | stages << 16 | kind << 24
     uint32_t round;
     uint16_t lane[32];
     uint16_t warp[1 << (kSortMaxThreadBits - 5)];
@@ -225,7 +273,8 @@ __device__ __forceinline__ void expand_groups(SortTab &tab, uint32_t cta, uint32
             g.head = make_uint4(G.code[0], G.code[1],
                                 ((uint32_t)G.reg[0] | (uint32_t)G.reg[1] << 16) << E_LOG,
                                 ((uint32_t)G.reg[2] | (uint32_t)G.reg[3] << 16) << E_LOG);
-            g.reg4 = (uint32_t)G.reg[4] << E_LOG | (uint32_t)G.n_stage << 16;
+            g.reg4 = (uint32_t)G.reg[4] << E_LOG | (uint32_t)G.n_stage << 16 |
+                     (uint32_t)G.kind << 24;
             g.round = (uint32_t)G.round << E_LOG;
         }
     }
@@ -294,7 +343,7 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
         const GroupTab &g = tab.grp[gi];
         const uint4 head = g.head;
         const uint32_t reg[3] = {head.z, head.w, g.reg4 & 0xffffu};
-        const uint32_t n_stage = g.reg4 >> 16, round = g.round;
+        const uint32_t n_stage = (g.reg4 >> 16) & 0xffu, kind = g.reg4 >> 24, round = g.round;
         const uint32_t base = (uint32_t)g.lane[lane] ^ g.warp[warp];
 #pragma unroll 1
         for (int rd = 0; rd < NR; ++rd) {
@@ -324,12 +373,15 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
                     run_stages<how, R>(n_stage, codes, v, u);
                 } else {
                     constexpr int how = KEY == dev::kKeyF32 ? kF32MinMax : dev::kKeyI64;
-                    run_stages<how, R>(n_stage, codes, v, u);
+                    if (kind) run_kind<how, R>(kind, v, u);
+                    else run_stages<how, R>(n_stage, codes, v, u);
                 }
                 if constexpr (KEY == dev::kKeyF64)
                     if (tab.d.last_pass && gi + 1 == n_group)
 #pragma unroll
                         for (int j = 0; j < E; ++j) v[j] = ordered(v[j]);
+            } else if (kind) {
+                run_kind<KEY, R>(kind, v, u);
             } else {
                 run_stages<KEY, R>(n_stage, codes, v, u);
             }

@@ -590,7 +590,17 @@ int build_groups(SortDesc *sd, const std::vector<uint64_t> &U, const std::vector
             if (group_coords(U, G, s, q, R, &tests, &codes)) e = q;
         if (e == s || !group_coords(U, G, s, e, R, &tests, &codes)) return -3;
         const int f = (int)tests.size();
-        Gr.n_stage = (uint16_t)(e - s);
+        Gr.n_stage = (uint8_t)(e - s);
+        for (int r = 0; r < f && e - s == f; ++r) {
+            bool cycle = true;
+            for (int q = 0; q < f; ++q) cycle &= codes[q] == sort_stage_code((r + q) % f, f);
+            if (cycle) Gr.kind = (uint8_t)sort_cycle_kind(f, r);
+        }
+        if (f == R && e - s == R * (R + 1) / 2) {
+            bool levels = true;
+            for (int q = 0; q < e - s; ++q) levels &= codes[q] == q;
+            if (levels) Gr.kind = (uint8_t)kSortLevelsKind;
+        }
         for (int q = 0; q < e - s; ++q) Gr.code[q / 8] |= (uint32_t)codes[q] << (4 * (q % 8));
         // vectors dual to the tests in the span of the partner vectors: the
         // stages' vectors, eliminated on the tests
@@ -663,10 +673,10 @@ int build_groups(SortDesc *sd, const std::vector<uint64_t> &U, const std::vector
 
 // Register bits of a thread.  Few keys per thread shorten the chain of a block's
 // instructions, many save round trips through shared memory: a whole sort in
-// one block of 2^11 keys runs in 12.7 us with 8 keys a thread and 14.6 with 16
-// (int32), 2^16 keys in 2^12-key blocks in 31 us with 16 and 33 with 32, and
-// 2^13-key blocks take 32 in their 13 stages' three groups.  32 8-byte keys do
-// not fit the registers.
+// one block of 2^11 keys takes 7.2 us with 8 keys a thread and 7.7 with 16
+// (int32; 9.8 and 11.3 int64), 2^18 keys in 2^12-key blocks 29.8 us with 16 and
+// 34.4 with 32 (int32), and 2^13-key blocks take 32 for their 13 stages in three
+// groups.  32 8-byte keys do not fit the registers.
 int reg_bits(int e_log, int D)
 {
     if (D <= 11) return 3;
@@ -831,9 +841,9 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
     // Default block: more keys per block are fewer passes, fewer keys are more
     // blocks and more threads per key.  The lines are where the larger block
     // starts to win (GB300, us, 2^12 / 2^13 / 2^14 4-byte keys: n = 18 float32
-    // 43 / 58 / 88, n = 20 74 / 72 / 113, n = 23 502 / 398 / 429, n = 24
-    // 1091 / 859 / 803; 2^12 / 2^13 8-byte keys: n = 22 int64 391 / 430,
-    // n = 23 857 / 806).
+    // 35 / 49 / 72, n = 20 66 / 64 / 95, n = 23 444 / 361 / 381, n = 24
+    // 984 / 805 / 721; 2^12 / 2^13 8-byte keys: n = 22 int64 355 / 383,
+    // n = 23 810 / 731).
     int D = block_log2 ? block_log2 - e_log : kMinBlockBits;
     if (!block_log2)
         D += e_log == 2 ? (N >= 20) + (N >= 24) : (N >= 23);
@@ -861,8 +871,9 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
         // combination of the bank bits, no choice of lanes avoids conflicts.
         // The vectors as they come leave half of the tests so in the passes that
         // start at the network's first stages; a few tries of random additions
-        // find layouts with none or nearly none (n = 24 float32, the 17 passes:
-        // 1482 us with the vectors as they come, 1161 us so).
+        // find layouts with none or nearly none (n = 24 float32, the 17 passes
+        // before the kernel's present form: 1482 us with the vectors as they come,
+        // 1161 us so).
         constexpr int kTries = 6;
         int best = -1;
         for (int attempt = 0; attempt < (last ? 1 : kTries) && best != 0; ++attempt) {
