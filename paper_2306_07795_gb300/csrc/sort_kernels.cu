@@ -43,8 +43,8 @@ __device__ __forceinline__ bool keep(V a, V b)
 // Float keys without NaN and -0.0 are totally ordered, and the pair may be
 // ordered by other means than IEEE <=: 4-byte ones by minimum and maximum, and
 // 8-byte ones, whose compare runs on the FP64 pipe at about two lanes a clock
-// per SM, as integers of the same order.  A block looks at its keys as it
-// first loads them and uses <= itself for the whole pass if any is special.
+// per SM, as integers of the same order.  A block looks at its keys as its
+// first group loads them and uses <= itself from then on if any is special.
 //
 // ordered(): the integer of a double's order, and back (its own inverse); the
 // order of signed integers is that of <= outside special keys, NaN beyond the
@@ -317,28 +317,15 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t n_group = tab.d.n_group;
     constexpr bool kFloat = KEY == dev::kKeyF32 || KEY == dev::kKeyF64;
-    bool exact = false;
-    if constexpr (kFloat && NR > 1) {  // the first group's keys are not all in registers at once
-        bool any = false;
-#pragma unroll 4
-        for (int c = 0; c < NR * E * (1 << E_LOG) / 16; ++c) {
-            uint4 *at = reinterpret_cast<uint4 *>(tile) + threadIdx.x + c * blockDim.x;
-            const uint4 w = *at;
-            if constexpr (KEY == dev::kKeyF32) {
-                any |= special<KEY>(w.x) || special<KEY>(w.y) || special<KEY>(w.z) || special<KEY>(w.w);
-            } else {
-                unsigned long long x = ((unsigned long long)w.y << 32) | w.x;
-                unsigned long long y = ((unsigned long long)w.w << 32) | w.z;
-                if (tab.d.first_pass) {
-                    x = ordered(x);
-                    y = ordered(y);
-                    *at = make_uint4((uint32_t)x, (uint32_t)(x >> 32), (uint32_t)y, (uint32_t)(y >> 32));
-                }
-                any |= special<KEY>(x) || special<KEY>(y);
-            }
-        }
-        exact = __syncthreads_or(any);
-    }
+    // Whether a key of the block is special is known after the first group's
+    // barrier; until then a warp goes by its own keys, since a pair's two are in
+    // one thread.  Asking the block before the first group's stages, or looking
+    // through the tile beforehand, costs a barrier (n = 24, the latter: float32
+    // 718 us against 692, float64 1763 against 1668); only where a thread has one
+    // set of 4-byte keys is the extra barrier cheaper than the warp's vote
+    // (n = 18 float32 32.3 against 33.3).
+    constexpr bool kAskBlock = KEY == dev::kKeyF32 && NR == 1;
+    bool exact = false, seen = false;
     for (uint32_t gi = 0; gi < n_group; ++gi) {
         const GroupTab &g = tab.grp[gi];
         const uint4 head = g.head;
@@ -355,7 +342,7 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
                 for (int j = 0; j < E; ++j) v[j] = *reinterpret_cast<const V *>(tile + at[j]);
             }
             uint64_t codes = ((uint64_t)head.y << 32) | head.x;
-            if constexpr (kFloat && NR == 1) {
+            if constexpr (kFloat) {
                 if (gi == 0) {
                     bool any = false;
 #pragma unroll
@@ -364,7 +351,8 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
                             if (tab.d.first_pass) v[j] = ordered(v[j]);
                         any |= special<KEY>(v[j]);
                     }
-                    exact = __syncthreads_or(any);
+                    exact = kAskBlock ? __syncthreads_or(any) : __any_sync(0xffffffffu, any);
+                    seen |= exact;
                 }
             }
             if constexpr (kFloat) {
@@ -395,7 +383,8 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
                 for (int j = 0; j < E; ++j) *reinterpret_cast<V *>(tile + at[j]) = v[j];
             }
         }
-        __syncthreads();
+        if (kFloat && !kAskBlock && gi == 0) exact = __syncthreads_or(seen);
+        else __syncthreads();
     }
 }
 
