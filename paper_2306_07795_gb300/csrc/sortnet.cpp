@@ -1099,6 +1099,10 @@ cudaError_t launch_sort_small(const SortSmallDesc &d, int e_log, const void *in,
 
 namespace {
 
+// Arrays of more than 2^12 keys take a workspace, also where one block holds
+// them and the one pass does not touch it.
+bool needs_workspace(const bmmc_sort_plan_s *p) { return p->N > 12; }
+
 bool overlaps(const void *a, const void *b, uint64_t bytes)
 {
     const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
@@ -1147,7 +1151,7 @@ int bmmc_sort_plan_num_passes(bmmc_sort_plan p)
 
 size_t bmmc_sort_workspace_bytes(bmmc_sort_plan p)
 {
-    if (!p || p->small || p->pass.size() < 2) return 0;
+    if (!p || !needs_workspace(p)) return 0;
     return ((size_t)1 << p->N) << p->e_log;
 }
 
@@ -1166,7 +1170,7 @@ int bmmc_sort_execute(bmmc_sort_plan p, const void *in, void *out, void *ws,
                                                                                  : BMMC_ERR_CUDA;
     }
     const size_t np = p->pass.size();
-    if (np >= 2) {
+    if (needs_workspace(p)) {
         if (!ws) return BMMC_ERR_INVALID;
         if (overlaps(ws, in, bytes) || overlaps(ws, out, bytes)) return BMMC_ERR_ALIAS;
     }
