@@ -1,9 +1,8 @@
 // sort_kernels.cu -- fused passes of the sorting network of Sec. 6.1.
 //
-// A fused pass is the tiled BMMC pass of Sec. 4.1 (tile load into swizzled
-// shared memory, barrier, 16-byte gathers and stores: dev::tile_load and
-// dev::tile_store of tile_body.cuh) with comparator stages run on the tile in
-// between.  The stages come in groups (sort_desc.h): for one group, every
+// A fused pass is the tiled BMMC pass of Sec. 4.1 (16-byte asynchronous copies
+// into swizzled shared memory, barrier, 16-byte gathers and stores) with
+// comparator stages run on the tile in between.  The stages come in groups (sort_desc.h): for one group, every
 // thread loads 2^R keys of the tile into registers, and each stage of the group
 // orders pairs of those registers, the pair's low position (index with
 // g_s . x = 0) receiving the smaller key (Sec. 6.1: a pair is kept when
@@ -44,7 +43,7 @@ __device__ __forceinline__ bool keep(V a, V b)
 // ordered by other means than IEEE <=: 4-byte ones by minimum and maximum, and
 // 8-byte ones, whose compare runs on the FP64 pipe at about two lanes a clock
 // per SM, as integers of the same order.  A block looks at its keys as its
-// first group loads them and uses <= itself from then on if any is special.
+// first group loads them and keeps the exact comparator if any is special.
 //
 // ordered(): the integer of a double's order, and back (its own inverse); the
 // order of signed integers is that of <= outside special keys, NaN beyond the
@@ -492,7 +491,17 @@ __device__ __forceinline__ void store_chunks(const SortTile &t, const uint32_t (
 
 // One block of at most 256 threads per tile of 2^P keys; a thread runs NR sets of
 // 2^R keys in turn in each group and moves as many in and out, in 16-byte
-// chunks.
+// chunks.  64 KiB tiles run as two sets per thread, three blocks per SM, rather
+// than 512 threads, two per SM (n = 24 float32, before the stages were straight
+// sequences: 804 against 940 us).
+//
+// What bounds it: in the exchanges the ALU pipe, which takes 1.5 of the 2.5
+// instructions of a float pair at half rate; between them loads, shared memory
+// and the group barriers, with 24 to 32 warps per SM to hide them (a 14-stage
+// pass of 2^24 floats: issue and ALU about half busy, DRAM at 22 % of its peak).
+// The 17 passes of that sort take 691 us, 3.3 TB/s in and out and 3.6 T
+// comparators a second (1510 us as 29 passes of four-stage groups with a variant
+// per orientation); 16 rows of 2^16 doubles 61 us (299); 2^11 integers 7.2 (20).
 template <int E_LOG, int KEY, int R, int NR>
 __global__ void __launch_bounds__(kMaxSortThreads, NR == 1 ? 4 : 3)
     bmmc_sort_pass(const __grid_constant__ SortDesc sd, const uint8_t *__restrict__ in,
