@@ -54,18 +54,29 @@ __device__ __forceinline__ unsigned long long ordered(unsigned long long x)
     return ((unsigned long long)(hi ^ (m & 0x7fffffffu)) << 32) | ((uint32_t)x ^ m);
 }
 
-// NaN or -0.0 (8-byte keys as ordered() gives them; there also the infinities
-// and negative numbers too small for the high word).
-template <int KEY>
-__device__ __forceinline__ bool special(uint32_t x)
+// Whether any of 2^R keys is special: NaN or -0.0 (8-byte keys as ordered() gives
+// them; there also the infinities and negative numbers too small for the high
+// word).  By the extremes of the keys' bits (8-byte keys: of the high words) as
+// signed and unsigned integers, two keys an instruction (n = 24: float32 692 -> 684 us
+// against two compares a key, float64 1658 -> 1647 against three operations).
+template <int E, typename V>
+__device__ __forceinline__ bool any_special(const V (&v)[E])
 {
-    return !(__uint_as_float(x) == __uint_as_float(x)) || x == 0x80000000u;
-}
-template <int KEY>
-__device__ __forceinline__ bool special(unsigned long long x)
-{
-    const uint32_t hi = (uint32_t)(x >> 32);
-    return hi - 0x80100000u >= 0x7ff00000u - 0x80100000u || hi == ~0u;
+    constexpr int kShift = sizeof(V) == 8 ? 32 : 0;
+    int32_t top = (int32_t)(v[0] >> kShift), low = top;
+    uint32_t utop = (uint32_t)top;
+#pragma unroll
+    for (int j = 1; j < E; j += 2) {
+        const uint32_t x = (uint32_t)(v[j] >> kShift);
+        const uint32_t y = j + 1 < E ? (uint32_t)(v[j + 1] >> kShift) : x;
+        top = __vimax3_s32(top, (int32_t)x, (int32_t)y);
+        low = __vimin3_s32(low, (int32_t)x, (int32_t)y);
+        utop = __vimax3_u32(utop, x, y);
+    }
+    if constexpr (sizeof(V) == 4)  // NaN: above the infinities; -0.0: the lowest
+        return top > 0x7f800000 || utop > 0xff800000u || low == (int32_t)0x80000000;
+    else  // -0.0 has the greatest high word of all, unsigned
+        return top >= 0x7ff00000 || low < (int32_t)0x80100000 || utop == ~0u;
 }
 
 // How a stage orders pairs: as the key type, or one of these.
@@ -356,13 +367,11 @@ __device__ __forceinline__ void run_groups(const SortTab &tab, uint8_t *tile, Un
             uint64_t codes = ((uint64_t)head.y << 32) | head.x;
             if constexpr (kFloat) {
                 if (gi == 0) {
-                    bool any = false;
+                    if constexpr (KEY == dev::kKeyF64)
+                        if (tab.d.first_pass)
 #pragma unroll
-                    for (int j = 0; j < E; ++j) {
-                        if constexpr (KEY == dev::kKeyF64)
-                            if (tab.d.first_pass) v[j] = ordered(v[j]);
-                        any |= special<KEY>(v[j]);
-                    }
+                            for (int j = 0; j < E; ++j) v[j] = ordered(v[j]);
+                    const bool any = any_special(v);
                     exact = kAskBlock ? __syncthreads_or(any) : __any_sync(0xffffffffu, any);
                     seen |= exact;
                 }
@@ -499,9 +508,9 @@ __device__ __forceinline__ void store_chunks(const SortTile &t, const uint32_t (
 // instructions of a float pair at half rate; between them loads, shared memory
 // and the group barriers, with 24 to 32 warps per SM to hide them (a 14-stage
 // pass of 2^24 floats: issue and ALU about half busy, DRAM at 22 % of its peak).
-// The 17 passes of that sort take 691 us, 3.3 TB/s in and out and 3.6 T
+// The 17 passes of that sort take 684 us, 3.3 TB/s in and out and 3.7 T
 // comparators a second (1510 us as 29 passes of four-stage groups with a variant
-// per orientation); 16 rows of 2^16 doubles 61 us (299); 2^11 integers 7.2 (20).
+// per orientation); 16 rows of 2^16 doubles 60 us (299); 2^11 integers 7.2 (20).
 template <int E_LOG, int KEY, int R, int NR>
 __global__ void __launch_bounds__(kMaxSortThreads, NR == 1 ? 4 : 3)
     bmmc_sort_pass(const __grid_constant__ SortDesc sd, const uint8_t *__restrict__ in,
