@@ -59,11 +59,12 @@ int bmmc_sort_plan_create(bmmc_sort_plan *out, int n, int b, int key_type,
 /* Release a plan.  NULL-safe. */
 void bmmc_sort_plan_destroy(bmmc_sort_plan p);
 
-/* Kernel launches one execution makes (1 for arrays of at most 2^12 keys). */
+/* Kernel launches one execution makes: 1 where a thread block holds the array,
+ * or a whole number of its rows (always up to 2^12 keys). */
 int bmmc_sort_plan_num_passes(bmmc_sort_plan p);
 
-/* Device workspace bmmc_sort_execute needs: one array of 2^(n + b) keys for
- * arrays of more than 2^12 keys, else 0.  0 for a NULL plan. */
+/* Device workspace bmmc_sort_execute needs: one array of 2^(n + b) keys for a
+ * plan of two passes or more, else 0.  0 for a NULL plan. */
 size_t bmmc_sort_workspace_bytes(bmmc_sort_plan p);
 
 /*

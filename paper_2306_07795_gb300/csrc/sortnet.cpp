@@ -1099,9 +1099,9 @@ cudaError_t launch_sort_small(const SortSmallDesc &d, int e_log, const void *in,
 
 namespace {
 
-// Arrays of more than 2^12 keys take a workspace, also where one block holds
-// them and the one pass does not touch it.
-bool needs_workspace(const bmmc_sort_plan_s *p) { return p->N > 12; }
+// Passes alternate between the output and a workspace; one alone writes the
+// output.
+bool needs_workspace(const bmmc_sort_plan_s *p) { return p->pass.size() > 1; }
 
 bool overlaps(const void *a, const void *b, uint64_t bytes)
 {

@@ -57,3 +57,25 @@ def test_groups(n, b, block_log2, dtype, special):
     B.bmmc_sort_plan_destroy(h)
     got = y.cpu().numpy().view(dtype)
     assert np.array_equal(got.view(np.uint8), want.view(np.uint8))
+
+
+@pytest.mark.parametrize("n,b", [(5, 10), (10, 6), (10, 10)])
+@pytest.mark.parametrize("dtype", [np.int32, np.uint64])
+def test_rows_without_workspace(n, b, dtype):
+    """Rows that fit a thread block are one pass: no workspace, and one that is
+    passed all the same is left alone."""
+    import torch
+    x = _keys(dtype, 1 << (n + b), None, n + b)
+    h = B.bmmc_sort_plan_create(n, b, KEYS[dtype])
+    assert B.bmmc_sort_workspace_bytes(h) == 0
+    d = torch.from_numpy(x.view(np.int32 if x.itemsize == 4 else np.int64).copy()).cuda()
+    y, z, ws = (torch.full_like(d, -1) for _ in range(3))
+    s = torch.cuda.current_stream().cuda_stream
+    B.bmmc_sort_execute(h, d.data_ptr(), y.data_ptr(), None, s)
+    B.bmmc_sort_execute(h, d.data_ptr(), z.data_ptr(), ws.data_ptr(), s)
+    torch.cuda.synchronize()
+    B.bmmc_sort_plan_destroy(h)
+    want = np.sort(x.reshape(1 << b, 1 << n), axis=1).reshape(-1)
+    assert np.array_equal(y.cpu().numpy().view(dtype), want)
+    assert torch.equal(y, z)
+    assert bool((ws == -1).all())

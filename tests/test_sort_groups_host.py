@@ -28,8 +28,25 @@ def test_block_sizes(key, least):
                 continue
             h = B.bmmc_sort_plan_create(n, 0, key, block_log2)
             e = 4 if key == B.BMMC_KEY_U32 else 8
-            assert B.bmmc_sort_workspace_bytes(h) == (0 if n <= 12 else e << n)
+            one = n <= 12 or e << n <= 1 << block_log2  # the block holds every key
+            assert (B.bmmc_sort_plan_num_passes(h) == 1) == one
+            assert B.bmmc_sort_workspace_bytes(h) == (0 if one else e << n)
             B.bmmc_sort_plan_destroy(h)
+
+
+@pytest.mark.parametrize("key,e", [(B.BMMC_KEY_F32, 4), (B.BMMC_KEY_U64, 8)])
+def test_workspace_of_rows(key, e):
+    """Rows that fit a thread block are one pass, however many they are, and
+    take no workspace; longer ones take one array."""
+    for n, b in ((1, 12), (5, 20), (10, 3), (10, 10), (1, 31), (12, 1), (13, 0), (14, 6), (16, 8)):
+        h = B.bmmc_sort_plan_create(n, b, key)
+        one = B.bmmc_sort_plan_num_passes(h) == 1
+        if n <= 10:
+            assert one
+        if n > 12:
+            assert not one
+        assert B.bmmc_sort_workspace_bytes(h) == (0 if one else e << (n + b))
+        B.bmmc_sort_plan_destroy(h)
 
 
 def test_fewest_passes():
