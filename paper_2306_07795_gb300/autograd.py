@@ -19,15 +19,20 @@ from .plan import Plan
 _lift_cache = {}
 
 
-def _lifted_plan(plan, rows_total):
-    b = rows_total.bit_length() - 1
-    if rows_total != 1 << b:
-        return None
+def _lifted_plan(plan, b):
+    """The plan lifted to 2^b rows, or None if there is none: the planner has no
+    tiles for long chosen segments in the longer array where it has some in one
+    row."""
     key = (id(plan), b)
     hit = _lift_cache.get(key)
     if hit is not None and hit[0] is plan:
         return hit[1]
-    lifted = plan.lift(b)
+    try:
+        lifted = plan.lift(b)
+    except B.BmmcError as err:
+        if err.code != B.BMMC_ERR_UNSUPPORTED:
+            raise
+        lifted = None
     _lift_cache[key] = (plan, lifted)
     return lifted
 
@@ -43,7 +48,9 @@ def _apply(plan, x):
     rows_total = x.numel() // x.shape[-1]
     # an odd count of groups of 2^b rows, each group one array of the lifted plan
     b = min((rows_total & -rows_total).bit_length() - 1, 32 - plan.n) if rows_total > 1 else 0
-    lifted = _lifted_plan(plan, 1 << b) if b else plan
+    lifted = _lifted_plan(plan, b) if b else plan
+    if lifted is None:
+        lifted, b = plan, 0
     groups = max(rows_total >> b, 1)
     out = lifted.run_rows(x, groups)
     if out is not None:

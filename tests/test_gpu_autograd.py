@@ -87,6 +87,27 @@ def test_non_power_of_two_rows_and_dtypes():
         assert torch.equal(x.grad, gy[:, :, dest])
 
 
+@pytest.mark.parametrize("n,seg_bits,rows_b", [(13, 12, 6), (13, 12, 4), (9, 8, 96), (9, 8, 32)])
+def test_rows_of_a_plan_that_cannot_be_lifted(n, seg_bits, rows_b):
+    """Long chosen segments: one row has tiles, 2^b rows as one array have none,
+    and the rows are permuted as they are (in one launch where the plan is one)."""
+    import torch
+    rows, c = wl.dense_bmmc(n, n, _inv)
+    plan = bm.Plan(n, rows, c, 16, seg_bits=seg_bits)
+    with pytest.raises(bm.BmmcError) as ei:
+        plan.lift((rows_b & -rows_b).bit_length() - 1)
+    assert ei.value.code == bm.BMMC_ERR_UNSUPPORTED
+    x = torch.randn(rows_b, 4 << n, device="cuda", requires_grad=True)
+    y = bmmc_permute(x, plan)
+    dest = torch.from_numpy(_dest_index(n, rows, c)).cuda()
+    want = torch.empty_like(x.detach()).view(rows_b, 1 << n, 4)
+    want[:, dest] = x.detach().view(rows_b, 1 << n, 4)
+    assert torch.equal(y.view_as(want), want)
+    gy = torch.randn_like(y)
+    y.backward(gy)
+    assert torch.equal(x.grad.view_as(want), gy.view_as(want)[:, dest])
+
+
 def test_gradcheck_small():
     import torch
     n = 6
