@@ -16,25 +16,19 @@ Any other count of rows is an odd count of such arrays, which share one launch.
 from . import _binding as B
 from .plan import Plan
 
-_lift_cache = {}
-
 
 def _lifted_plan(plan, b):
     """The plan lifted to 2^b rows, or None if there is none: the planner has no
     tiles for long chosen segments in the longer array where it has some in one
-    row."""
-    key = (id(plan), b)
-    hit = _lift_cache.get(key)
-    if hit is not None and hit[0] is plan:
-        return hit[1]
-    try:
-        lifted = plan.lift(b)
-    except B.BmmcError as err:
-        if err.code != B.BMMC_ERR_UNSUPPORTED:
-            raise
-        lifted = None
-    _lift_cache[key] = (plan, lifted)
-    return lifted
+    row.  Kept by the plan, and released with it."""
+    if b not in plan.lifts:
+        try:
+            plan.lifts[b] = plan.lift(b)
+        except B.BmmcError as err:
+            if err.code != B.BMMC_ERR_UNSUPPORTED:
+                raise
+            plan.lifts[b] = None
+    return plan.lifts[b]
 
 
 def _apply(plan, x):

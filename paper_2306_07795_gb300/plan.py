@@ -55,6 +55,7 @@ class Plan:
                                             self.elem_bytes, flags, seg_bits,
                                             cta_tile_log2, tile_order)
         self._inverse = None
+        self.lifts = {}  # b -> the plan lifted to 2^b rows (see autograd)
         self._ws_bytes = None
         self._nbytes = (1 << self.n) * self.elem_bytes
         # plans are immutable: what a call needs of the library, looked up once

@@ -2,11 +2,15 @@
 do, and that the launch moves every element as the two passes, or the launches
 row by row, do."""
 
+import gc
+import weakref
+
 import pytest
 
 import oracle
 from oracle import f2
 import paper_2306_07795_gb300 as bm
+from paper_2306_07795_gb300.autograd import _lifted_plan
 import workloads as wl
 
 
@@ -35,6 +39,18 @@ def test_rule(e, n):
     assert (q.num_passes, q.num_launches) == (2, 2)
     assert q.pass_matrices() == p.pass_matrices()
     assert q.verify() == 0
+
+
+def test_lifted_plans_go_with_their_plan():
+    """A program that makes a plan per call keeps none of their lifted forms."""
+    rows, c = _dense(10, 4)
+    p = bm.Plan(10, rows, c, 4)
+    lifted = _lifted_plan(p, 3)
+    assert lifted is _lifted_plan(p, 3) and lifted.n == 13
+    refs = [weakref.ref(p), weakref.ref(lifted)]
+    del p, lifted
+    gc.collect()
+    assert [r() for r in refs] == [None, None]
 
 
 @pytest.mark.gpu
