@@ -7,8 +7,11 @@ paper's n_tile) and the bytes per thread block (cta_tile_log2) trade DRAM
 locality against occupancy on a given GPU and array size; this module times
 candidates on the device and keeps the fastest.
 
-Results for single plans are cached in a JSON file keyed by
-(n, element bytes, strategy, passes), so a size class is tuned once.
+A two-pass plan runs as one launch with the default segments and as two with
+chosen ones, so the candidates hold block sizes with either.
+
+Results for single plans are cached in a JSON file keyed by a version of the
+candidates and (n, element bytes, strategy, passes), so a size class is tuned once.
 """
 
 import json
@@ -21,9 +24,12 @@ from .plan import Plan
 # (seg_bits, cta_tile_log2); 0 = the planner's default
 DEFAULT = (0, 0)
 CANDIDATES = {
-    4: [(0, 0), (5, 13), (5, 14), (6, 13), (6, 15), (7, 15), (7, 16)],
-    8: [(0, 0), (4, 13), (4, 14), (5, 13), (5, 15), (6, 15), (6, 16)],
-    16: [(0, 0), (3, 13), (3, 14), (4, 13), (4, 15), (5, 15), (5, 16)],
+    4: [(0, 0), (0, 13), (0, 15), (0, 16),
+        (5, 13), (5, 14), (6, 13), (6, 15), (7, 15), (7, 16)],
+    8: [(0, 0), (0, 13), (0, 15), (0, 16),
+        (4, 13), (4, 14), (5, 13), (5, 15), (6, 15), (6, 16)],
+    16: [(0, 0), (0, 13), (0, 15), (0, 16),
+         (3, 13), (3, 14), (4, 13), (4, 15), (5, 15), (5, 16)],
 }
 
 
@@ -63,6 +69,10 @@ def tune_batch(make_batch, dev, candidates=None, reps=3):
 class TuneCache:
     """JSON-backed cache of tuned plan options."""
 
+    # In the key: entries timed when two-pass plans always were two launches
+    # name segments that would take the one launch away.
+    VERSION = 2
+
     def __init__(self, path=None):
         self.path = path or os.environ.get(
             "BMMC_TUNE_CACHE",
@@ -74,9 +84,9 @@ class TuneCache:
         except (OSError, ValueError):
             self.data = {}
 
-    @staticmethod
-    def key(n, e, flags, passes):
-        return "%d/%d/%d/%d" % (n, e, flags, passes)
+    @classmethod
+    def key(cls, n, e, flags, passes):
+        return "v%d/%d/%d/%d/%d" % (cls.VERSION, n, e, flags, passes)
 
     def get(self, n, e, flags, passes):
         v = self.data.get(self.key(n, e, flags, passes))

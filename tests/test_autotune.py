@@ -2,6 +2,7 @@
 candidate from its list, cached by size class, and plans built with it stay
 bit-exact."""
 
+import json
 import os
 
 import numpy as np
@@ -42,6 +43,23 @@ def test_candidates_plan_on_the_host():
         for seg, tile in cands:
             p = bm.Plan(18, rows, c, e, seg_bits=seg, cta_tile_log2=tile)
             assert p.verify() == 0
+
+
+def test_entries_of_two_launches_are_not_taken(tmp_path):
+    path = str(tmp_path / "tune.json")
+    with open(path, "w") as f:
+        json.dump({"20/4/0/2": [6, 15]}, f)
+    assert autotune.TuneCache(path).get(20, 4, 0, 2) is None
+
+
+def test_candidates_with_one_launch():
+    """Block sizes other than the default are tried without giving up the one
+    launch of a general matrix."""
+    rows, c = wl.dense_bmmc(20, 3, _inv)
+    for e, cands in autotune.CANDIDATES.items():
+        one = {tile for seg, tile in cands
+               if bm.Plan(20, rows, c, e, seg_bits=seg, cta_tile_log2=tile).num_launches == 1}
+        assert {0, 13, 15, 16} <= one
 
 
 @pytest.mark.gpu
