@@ -190,19 +190,21 @@ size_t bmmc_plan_workspace_bytes(bmmc_plan p);
  * in, out  device buffers of 2^n * elem_bytes bytes (see conventions).
  * stream   CUDA stream to run on.
  *
- * A two-pass plan has a workspace of bmmc_plan_workspace_bytes bytes; on
- * its first execution here the plan allocates one (cudaMalloc) and keeps
- * it until bmmc_plan_destroy (bmmc_execute_direct needs none).  Because that workspace is shared, at most one
- * execution of a given plan may be in flight at a time with this entry
- * point; use bmmc_execute_ws with distinct workspaces for concurrent
- * executions of one plan.
+ * A plan of two launches (bmmc_plan_num_launches) needs a workspace of
+ * bmmc_plan_workspace_bytes bytes; on its first execution here the plan
+ * allocates one (cudaMalloc) and keeps it until bmmc_plan_destroy.  Because
+ * that workspace is shared, at most one execution of such a plan may be in
+ * flight at a time with this entry point; use bmmc_execute_ws with distinct
+ * workspaces for concurrent executions of one plan.  A plan of one launch
+ * allocates nothing, and its executions may overlap.
  * Errors: INVALID, ALIAS, ALIGN, OOM, CUDA.
  */
 int bmmc_execute(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream);
 
 /* As bmmc_execute, with a caller-owned device workspace of at least
  * bmmc_plan_workspace_bytes(p) bytes (16-byte aligned, overlapping neither
- * in nor out).  ws may be NULL for a one-pass plan.
+ * in nor out).  ws may be NULL for a one-pass plan only: a two-pass plan whose
+ * passes run as one launch is refused without one, although it is not touched.
  * Errors: INVALID, ALIAS, ALIGN, CUDA. */
 int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws,
                     bmmc_stream_t stream);
@@ -229,8 +231,8 @@ int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, uint64_t rows,
  *                    streams.  host_out holds the result once `stream` has
  *                    reached the end of this call's work.
  * dev_in, dev_out    caller-owned device staging buffers (conventions above).
- * ws                 as for bmmc_execute_ws; NULL selects the plan-owned
- *                    workspace of bmmc_execute for a two-pass plan.
+ * ws                 as for bmmc_execute_ws; NULL runs the plan as
+ *                    bmmc_execute does (plan-owned workspace).
  * Calls on different streams with different staging buffers overlap: the
  * upload of one call runs beside the kernels of another and the download
  * of a third.

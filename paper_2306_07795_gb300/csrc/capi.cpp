@@ -180,16 +180,16 @@ int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
     return BMMC_OK;
 }
 
-// key: comparator epilogue of the last pass (0 = none).  A two-pass plan is
-// refused without a workspace, also when its one launch would not touch it.
-int execute_impl(bmmc_plan p, const void *in, void *out, void *ws, cudaStream_t s,
-                 int key = 0)
+// ws: used by plans of two launches.  takes_ws: refuse a missing or bad one.
+// key: comparator epilogue of the last pass (0 = none).
+int execute_impl(bmmc_plan p, const void *in, void *out, void *ws, bool takes_ws,
+                 cudaStream_t s, int key = 0)
 {
     const uint64_t bytes = array_bytes(p);
     if (p->derived < p->npass) return BMMC_ERR_INVALID;
     if (((uintptr_t)in | (uintptr_t)out) & 15u) return BMMC_ERR_ALIGN;
     if (overlap(in, out, bytes)) return BMMC_ERR_ALIAS;
-    if (p->npass == 2) {
+    if (takes_ws) {
         if (!ws) return BMMC_ERR_INVALID;
         if ((uintptr_t)ws & 15u) return BMMC_ERR_ALIGN;
         if (overlap(ws, in, bytes) || overlap(ws, out, bytes)) return BMMC_ERR_ALIAS;
@@ -373,7 +373,8 @@ int bmmc_execute(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream)
 {
     if (!p || !in || !out) return BMMC_ERR_INVALID;
     void *ws = nullptr;
-    if (p->npass == 2) {
+    const bool two = p->launches() == 2;
+    if (two) {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return BMMC_ERR_CUDA;
         std::lock_guard<std::mutex> lock(p->ws_mu);
@@ -389,13 +390,15 @@ int bmmc_execute(bmmc_plan p, const void *in, void *out, bmmc_stream_t stream)
         }
         ws = p->ws;
     }
-    return execute_impl(p, in, out, ws, (cudaStream_t)stream);
+    return execute_impl(p, in, out, ws, two, (cudaStream_t)stream);
 }
 
 int bmmc_execute_ws(bmmc_plan p, const void *in, void *out, void *ws, bmmc_stream_t stream)
 {
+    // Every two-pass plan takes a workspace here, as its workspace_bytes says,
+    // also one whose single launch would not touch it.
     if (!p || !in || !out) return BMMC_ERR_INVALID;
-    return execute_impl(p, in, out, ws, (cudaStream_t)stream);
+    return execute_impl(p, in, out, ws, p->npass == 2, (cudaStream_t)stream);
 }
 
 int bmmc_execute_direct(bmmc_plan p, const void *in, void *out, uint64_t rows,
@@ -425,7 +428,7 @@ int bmmc_execute_host(bmmc_plan p, const void *host_in, void *host_out, void *de
     if (cudaMemcpyAsync(dev_in, host_in, (size_t)bytes, cudaMemcpyHostToDevice, s) !=
         cudaSuccess)
         return BMMC_ERR_CUDA;
-    const int rc = ws ? execute_impl(p, dev_in, dev_out, ws, s)
+    const int rc = ws ? execute_impl(p, dev_in, dev_out, ws, p->npass == 2, s)
                       : bmmc_execute(p, dev_in, dev_out, stream);
     if (rc != BMMC_OK) return rc;
     if (cudaMemcpyAsync(host_out, dev_out, (size_t)bytes, cudaMemcpyDeviceToHost, s) !=
@@ -442,7 +445,7 @@ int bmmc_execute_ce(bmmc_plan p, const void *in, void *out, void *ws, int key_ty
     const bool ok8 = p->e_log == 3 && key_type >= BMMC_KEY_I64 && key_type <= BMMC_KEY_F64;
     if (!ok4 && !ok8) return BMMC_ERR_UNSUPPORTED;
     if (p->n < 1) return BMMC_ERR_UNSUPPORTED;
-    return execute_impl(p, in, out, ws, (cudaStream_t)stream, key_type);
+    return execute_impl(p, in, out, ws, p->npass == 2, (cudaStream_t)stream, key_type);
 }
 
 int bmmc_device_wait_timeouts(unsigned long long *count)

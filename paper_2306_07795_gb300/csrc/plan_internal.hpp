@@ -35,7 +35,7 @@ struct bmmc_plan_s {
     bmmc::PassInfo whole_info;
     std::mutex derive_mu;
     bool factors_derived = false;
-    // Workspace owned by the plan for bmmc_execute (two-pass plans only).
+    // Workspace owned by the plan for bmmc_execute (plans of two launches only).
     std::mutex ws_mu;
     void *ws = nullptr;
     int ws_device = -1;

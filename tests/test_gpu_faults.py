@@ -34,8 +34,8 @@ def _dense(n=18, e=4, seed=3):
 def test_plan_owned_workspace_allocation_failure():
     import torch
     n, e, rows, c = _dense()
-    p = bm.Plan(n, rows, c, e)
-    assert p.num_passes == 2
+    p = bm.Plan(n, rows, c, e, seg_bits=6)  # chosen segments: two launches
+    assert p.num_launches == 2
     x = torch.arange(1 << n, dtype=torch.int32, device="cuda")
     y = torch.empty_like(x)
     s = torch.cuda.current_stream().cuda_stream
@@ -48,6 +48,26 @@ def test_plan_owned_workspace_allocation_failure():
     torch.cuda.synchronize()
     want = oracle.apply(n, rows, c, np.arange(1 << n, dtype=np.uint32))
     assert np.array_equal(y.cpu().numpy().view(np.uint32), want)
+
+
+def test_one_launch_allocates_no_workspace():
+    """A two-pass plan that runs as one launch: bmmc_execute allocates nothing
+    (an allocation would fail here), and executions of one plan may overlap."""
+    import torch
+    n, e, rows, c = _dense(20)
+    p = bm.Plan(n, rows, c, e)
+    assert (p.num_passes, p.num_launches) == (2, 1)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    xs = [torch.arange(i, i + (1 << n), dtype=torch.int32, device="cuda") for i in range(3)]
+    ys = [torch.empty_like(x) for x in xs]
+    torch.cuda.synchronize()
+    bm.bmmc_debug_fail_allocs(1)
+    for x, y, s in zip(xs, ys, streams):
+        bm.bmmc_execute(p.handle, x.data_ptr(), y.data_ptr(), s.cuda_stream)
+    torch.cuda.synchronize()
+    for i, y in enumerate(ys):
+        want = oracle.apply(n, rows, c, np.arange(i, i + (1 << n), dtype=np.uint32))
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), want)
 
 
 @pytest.mark.parametrize("passes", [1, 2])

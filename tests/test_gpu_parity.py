@@ -157,13 +157,14 @@ def test_inverse_round_trip_and_repeatability():
     assert torch.equal(back, x)
 
 
-def test_plan_owned_workspace_entry_point():
+@pytest.mark.parametrize("seg_bits,launches", [(0, 1), (6, 2)])
+def test_plan_owned_workspace_entry_point(seg_bits, launches):
     """bmmc_execute (plan-owned workspace) agrees with bmmc_execute_ws."""
     import torch
     n = 19
     rows, c = wl.dense_bmmc(n, 31, oracle_invertible)
-    p = bm.Plan(n, rows, c, 4)
-    assert p.num_passes == 2
+    p = bm.Plan(n, rows, c, 4, seg_bits=seg_bits)
+    assert (p.num_passes, p.num_launches) == (2, launches)
     x = to_device(wl.payload(n, 4))
     out = torch.empty_like(x)
     bm.bmmc_execute(p.handle, x.data_ptr(), out.data_ptr(),
