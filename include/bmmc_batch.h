@@ -5,11 +5,11 @@
  * All first passes of the batch (the whole permutation for a plan of one
  * launch, see bmmc_plan_num_launches; (R L P, 0) of Sec. 5.2 for the others)
  * run as one launch per element size present; the second passes ((U R, c)) of
- * the others run as a second such launch.  Each launch is a persistent grid of (SMs x resident blocks) thread
- * blocks that take chunks of consecutive tiles of the batch, so many small
- * arrays, which cannot fill the GPU one at a time (Sec. 6, arrays under 2^20
- * elements), share the machine, and a batch of any size costs at most six
- * launches.  The launches read the tables uploaded at creation and update
+ * the others run as a second such launch.  Each launch is a persistent grid of
+ * (SMs x resident blocks) thread blocks that take chunks of consecutive tiles
+ * of the batch, so many small arrays, which cannot fill the GPU one at a time
+ * (Sec. 6, arrays under 2^20 elements), share the machine, and a batch of any
+ * size costs at most six launches.  The launches read the tables uploaded at creation and update
  * two chunk counters per launch in the same memory (each launch leaves them
  * at zero when it ends), so the launches of one batch must not overlap one
  * another (they write the same outputs anyway).
@@ -28,13 +28,13 @@ extern "C" {
 
 typedef struct bmmc_batch_s *bmmc_batch;
 
-/* Device workspace bytes a batch of these plans needs: the sum over the
- * two-pass plans of 2^n * elem_bytes, each slice starting on a 256-byte
- * boundary.  0 if every plan has one pass or the arguments are invalid. */
+/* Device workspace bytes a batch of these plans needs: the sum over the plans
+ * of two launches of 2^n * elem_bytes, each slice starting on a 256-byte
+ * boundary.  0 if every plan is one launch or the arguments are invalid. */
 size_t bmmc_batch_workspace_bytes(const bmmc_plan *plans, int count);
 
 /* Device bytes of a batch's tables (bmmc_batch_create's `table`): about
- * 1.4 KB per pass plus 32 bytes per pass, plus 96 bytes of counters.  0 for
+ * 1.4 KB per launch of each plan plus 32 bytes, plus 96 bytes of counters.  0 for
  * invalid arguments. */
 size_t bmmc_batch_table_bytes(const bmmc_plan *plans, int count);
 
@@ -84,7 +84,7 @@ void bmmc_batch_destroy(bmmc_batch b);
 
 /*
  * One-shot form: run plans[i] on ins[i] -> outs[i] for i < count as one batch
- * on `stream`, with the tables and the two-pass workspace taken from the
+ * on `stream`, with the tables and the workspace taken from the
  * stream-ordered allocator (cudaMallocAsync) and given back (cudaFreeAsync)
  * on the same stream, so the call never synchronises the device.  Equivalent
  * to create, execute and destroy with memory that lives exactly as long as

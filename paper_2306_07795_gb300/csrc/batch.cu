@@ -5,8 +5,9 @@
 // thread-block items of every pass: phase 1 holds the first pass of every
 // plan (in -> out for plans of one launch, in -> workspace slice for the
 // others), phase 2 the second pass of the latter (workspace -> out,
-// Sec. 5.2).  Each phase is one persistent kernel per element size present: a grid of (SMs x resident blocks) thread blocks, each walking a contiguous
-// range of items, so that small arrays (the paper notes that arrays under
+// Sec. 5.2).  Each phase is one persistent kernel per element size present: a
+// grid of (SMs x resident blocks) thread blocks that take chunks of
+// consecutive items, so that small arrays (the paper notes that arrays under
 // 2^20 elements cannot fill a GPU, Sec. 6) share the machine with large ones
 // instead of each needing its own launch.  A block reloads a pass's tables
 // into shared memory only when its range crosses into the next array.
@@ -343,14 +344,14 @@ namespace {
 constexpr int kMaxGroups = 6;
 constexpr size_t kCounterBytes = 16;  // per group: claims, finished blocks
 
-// Bytes of the device tables of a batch: one 128-byte slot per pass, then
-// one BatchEntry per (array, pass), then the chunk counters of each group.
+// Bytes of the device tables of a batch: one slot per launch of each plan, then
+// one BatchEntry for each, then the chunk counters of each group.
 size_t table_bytes(const bmmc_plan *plans, int count)
 {
-    size_t passes = 0;
+    size_t launches = 0;
     for (int i = 0; i < count; ++i)
-        if (plans[i]) passes += (size_t)plans[i]->npass;
-    return passes * kDescSlot + passes * sizeof(BatchEntry) + kMaxGroups * kCounterBytes;
+        if (plans[i]) launches += (size_t)plans[i]->launches();
+    return launches * kDescSlot + launches * sizeof(BatchEntry) + kMaxGroups * kCounterBytes;
 }
 
 int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
@@ -367,7 +368,7 @@ size_t bmmc_batch_workspace_bytes(const bmmc_plan *plans, int count)
     if (!plans || count <= 0) return 0;
     uint64_t total = 0;
     for (int i = 0; i < count; ++i)
-        if (plans[i] && plans[i]->npass == 2) total = round_up(total, 256) + plans[i]->bytes();
+        if (plans[i] && plans[i]->launches() == 2) total = round_up(total, 256) + plans[i]->bytes();
     return (size_t)total;
 }
 
@@ -460,7 +461,7 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
     if (ws_need && !ws) return BMMC_ERR_INVALID;
     if ((uintptr_t)ws & 15u) return BMMC_ERR_ALIGN;
 
-    // Workspace slices and overlap checks.
+    // Workspace slices (of the plans of two launches) and overlap checks.
     std::vector<uint8_t *> slice(count, nullptr);
     std::vector<Range> ranges;
     ranges.reserve(3 * (size_t)count);
@@ -472,7 +473,7 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
         const uint64_t b = p->bytes();
         ranges.push_back({(uintptr_t)ins[i], (uintptr_t)ins[i] + b, false});
         ranges.push_back({(uintptr_t)outs[i], (uintptr_t)outs[i] + b, true});
-        if (p->npass == 2) {
+        if (p->launches() == 2) {
             off = round_up(off, 256);
             slice[i] = (uint8_t *)ws + off;
             ranges.push_back({(uintptr_t)slice[i], (uintptr_t)slice[i] + b, true});
@@ -481,7 +482,7 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
     }
     if (ranges_conflict(ranges)) return BMMC_ERR_ALIAS;
 
-    // Pass tables: one slot per (plan, pass).
+    // Pass tables: one slot per launch of each plan.
     std::vector<uint32_t> desc0(count), desc1(count);
     uint32_t ndesc = 0;
     for (int i = 0; i < count; ++i) {

@@ -41,6 +41,16 @@ def test_rule(e, n):
     assert q.verify() == 0
 
 
+def test_batch_workspace():
+    """Only plans of two launches have a slice of a batch's workspace."""
+    rows, c = _dense(18, 2)
+    one = [bm.Plan(18, rows, c, 4), bm.Plan(18, wl.bit_reverse(18), 0, 4),
+           bm.Plan(18, rows, c, 8, flags=bm.BMMC_PLAN_SINGLE_PASS)]
+    two = bm.Plan(18, rows, c, 4, seg_bits=6)
+    assert bm.bmmc_batch_workspace_bytes([p.handle for p in one]) == 0
+    assert bm.bmmc_batch_workspace_bytes([p.handle for p in one + [two]]) == two.nbytes
+
+
 def test_lifted_plans_go_with_their_plan():
     """A program that makes a plan per call keeps none of their lifted forms."""
     rows, c = _dense(10, 4)

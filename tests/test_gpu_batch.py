@@ -30,12 +30,13 @@ def _case(i, n, e, seed):
     return wl.tiled_only_bmmc(n, k, seed, _inv)
 
 
-def _build(ns, es, flags, seed0=0):
+def _build(ns, es, flags, seed0=0, two_launches=()):
     import torch
     plans, ins, outs, host = [], [], [], []
     for i, (n, e) in enumerate(zip(ns, es)):
         rows, c = _case(i, n, e, seed0 + i)
-        plans.append(bm.Plan(n, rows, c, e, flags=flags))
+        seg_bits = 8 - (e.bit_length() - 1) if i in two_launches else 0
+        plans.append(bm.Plan(n, rows, c, e, flags=flags, seg_bits=seg_bits))
         arr = wl.payload(n, e, seed=i)
         host.append((n, e, rows, c, arr))
         flat = np.ascontiguousarray(arr).reshape(-1).view(np.int32)
@@ -216,3 +217,25 @@ def test_one_shot_execute_batch():
     with pytest.raises(bm.BmmcError) as ei:
         bm.bmmc_execute_batch([], [], [], 0)
     assert ei.value.code == bm.BMMC_ERR_INVALID
+
+
+def test_plans_of_one_and_two_launches():
+    """A batch whose general matrices run as one launch (no slice of the
+    workspace) beside others of two (chosen segments: a slice each)."""
+    import torch
+    ns = [18, 19, 15, 17, 16, 20, 12, 19]
+    es = [4, 8, 16, 4, 8, 4, 4, 16]
+    plans, ins, outs, host = _build(ns, es, bm.BMMC_PLAN_PAPER, seed0=90, two_launches=(4, 5))
+    assert [p.num_launches for p in plans] == [1, 1, 1, 1, 2, 2, 1, 1]
+    b = Batch(plans, ins, outs)
+    assert b.workspace.numel() == plans[4].nbytes + plans[5].nbytes
+    for _ in range(3):
+        b()
+    torch.cuda.synchronize()
+    _check(outs, host)
+    for y in outs:
+        y.fill_(-1)
+    bm.bmmc_execute_batch([p.handle for p in plans], [x.data_ptr() for x in ins],
+                          [y.data_ptr() for y in outs], torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    _check(outs, host)
