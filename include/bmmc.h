@@ -249,10 +249,11 @@ int bmmc_execute_host(bmmc_plan p, const void *host_in, void *host_out, void *de
  * block and synchronise the device, and programs that must fix their peak
  * device memory in advance.
  *
- * A two-pass plan keeps its intermediate array in one file-scope device array
- * of BMMC_STATIC_SCRATCH_BYTES bytes, reserved on every GPU that loads the
- * library's device code and held until the process exits.  A one-pass plan
- * needs no intermediate array and runs exactly as with bmmc_execute_ws.
+ * A plan of two launches keeps its intermediate array in one file-scope device
+ * array of BMMC_STATIC_SCRATCH_BYTES bytes, reserved on every GPU that loads
+ * the library's device code and held until the process exits.  A plan of one
+ * launch needs no intermediate array, has no limit of size here and runs
+ * exactly as with bmmc_execute; what follows is about the others.
  *
  * in, out, stream: as for bmmc_execute.
  * Each call looks up the array's device address in the current context
@@ -268,8 +269,8 @@ int bmmc_execute_host(bmmc_plan p, const void *host_in, void *host_out, void *de
  * calls whose executions overlap on the GPU (different streams, not ordered
  * by events) race on it and give wrong results.  Order such calls.
  * Errors: INVALID, ALIAS, ALIGN, CUDA, OOM (the array could not be loaded),
- * UNSUPPORTED (device index 64 or above), and TOO_LARGE when the plan's
- * workspace (2^n * elem_bytes) exceeds BMMC_STATIC_SCRATCH_BYTES.  The call
+ * UNSUPPORTED (device index 64 or above), and TOO_LARGE when the workspace of
+ * a plan of two launches (2^n * elem_bytes) exceeds BMMC_STATIC_SCRATCH_BYTES.  The call
  * itself never allocates or frees device memory.
  */
 #define BMMC_STATIC_SCRATCH_BYTES (32u << 20)

@@ -1,7 +1,7 @@
-// static_scratch.cu -- two-pass execution that allocates no device memory.
+// static_scratch.cu -- two-launch execution that allocates no device memory.
 //
-// A plan that needs two passes (Sec. 5.2) writes its first pass into an
-// intermediate array as large as the input.  bmmc_execute allocates that
+// A plan that runs as two launches (Sec. 5.2) writes its first pass into an
+// intermediate array as large as the input; any other needs none.  bmmc_execute allocates that
 // array on first use and bmmc_execute_ws takes it from the caller; both
 // assume somebody can allocate device memory.  Some callers cannot:
 //   * code that runs inside a host application which owns all device memory
@@ -79,9 +79,9 @@ extern "C" int bmmc_execute_static_ws(bmmc_plan p, const void *in, void *out,
 {
     return bmmc::guarded([&] {
         if (!p || !in || !out) return (int)BMMC_ERR_INVALID;
-        const size_t need = bmmc_plan_workspace_bytes(p);
-        if (need == 0) return bmmc_execute_ws(p, in, out, nullptr, stream);
-        if (need > (size_t)BMMC_STATIC_SCRATCH_BYTES) return (int)BMMC_ERR_TOO_LARGE;
+        // one launch needs no scratch, and bmmc_execute allocates nothing for it
+        if (bmmc_plan_num_launches(p) == 1) return bmmc_execute(p, in, out, stream);
+        if (bmmc_plan_workspace_bytes(p) > (size_t)BMMC_STATIC_SCRATCH_BYTES) return (int)BMMC_ERR_TOO_LARGE;
         void *ws = nullptr;
         int rc = scratch_address((cudaStream_t)stream, &ws);
         if (rc != BMMC_OK) return rc;

@@ -2,13 +2,14 @@
 
 Callers that may not allocate device memory (a host application that owns
 all of it, a latency-critical loop where cudaMalloc could stall, a program
-with a fixed memory budget) run two-pass plans through this entry point,
-which keeps the intermediate array in a static device array instead of
-allocating one.  These tests call it through the C ABI and require results
-identical, byte for byte, to bmmc_execute_ws with a caller workspace and to
-the CPU oracle, on two calls in a row (the second call reuses the array the
-first one left behind), and check that a call leaves the device's free memory
-unchanged.
+with a fixed memory budget) run plans of two launches through this entry
+point, which keeps the intermediate array in a static device array instead of
+allocating one.  These tests call it through the C ABI, with chosen segments
+(two launches through the array) and without (one launch that needs none), and
+require results identical, byte for byte, to bmmc_execute_ws with a caller
+workspace and to the CPU oracle, on two calls in a row (the second call reuses
+the array the first one left behind), and check that a call leaves the device's
+free memory unchanged.
 
 The file is named to be collected last, so that a run stopping at the first
 failure has run every other test before it.
@@ -59,15 +60,21 @@ def _static(plan, x):
     return out
 
 
+def _seg_bits(e, launches):
+    """Chosen segments (the default's size) make a two-pass plan two launches."""
+    return 0 if launches == 1 else 8 - (e.bit_length() - 1)
+
+
+@pytest.mark.parametrize("launches", [1, 2])
 @pytest.mark.parametrize("n,e", [(20, 4), (19, 8), (21, 16)])
-def test_static_scratch_matches_workspace_entry_point(n, e):
+def test_static_scratch_matches_workspace_entry_point(n, e, launches):
     import torch
     # two different dense BMMCs, each a two-pass plan, one call after the other
     plans = []
     for seed in (11, 12):
         rows, c = wl.dense_bmmc(n, seed, _inv)
-        p = bm.Plan(n, rows, c, e)
-        assert p.num_passes == 2
+        p = bm.Plan(n, rows, c, e, seg_bits=_seg_bits(e, launches))
+        assert (p.num_passes, p.num_launches) == (2, launches)
         assert 0 < p.workspace_bytes <= bm.BMMC_STATIC_SCRATCH_BYTES
         plans.append(p)
     xs = [_device_payload(n, e, seed=s) for s in (1, 2)]
@@ -88,14 +95,15 @@ def test_static_scratch_matches_workspace_entry_point(n, e):
         assert bad == 0, bad
 
 
-def test_static_scratch_allocates_nothing():
+@pytest.mark.parametrize("launches", [1, 2])
+def test_static_scratch_allocates_nothing(launches):
     """After a first call (which may load the library's device code), a
     two-pass call leaves the device's free memory exactly as it was."""
     import torch
     n, e = 20, 4
     rows, c = wl.dense_bmmc(n, 13, _inv)
-    p = bm.Plan(n, rows, c, e)
-    assert p.num_passes == 2
+    p = bm.Plan(n, rows, c, e, seg_bits=_seg_bits(e, launches))
+    assert (p.num_passes, p.num_launches) == (2, launches)
     x = _device_payload(n, e, seed=5)
     _static(p, x)
     torch.cuda.synchronize()
@@ -138,7 +146,8 @@ def test_static_scratch_rejects_oversize_plans():
     import torch
     n, e = 22, 16  # workspace 64 MiB > 32 MiB
     rows, c = wl.dense_bmmc(n, 5, _inv)
-    p = bm.Plan(n, rows, c, e)
+    p = bm.Plan(n, rows, c, e, seg_bits=_seg_bits(e, 2))
+    assert p.num_launches == 2
     assert p.workspace_bytes > bm.BMMC_STATIC_SCRATCH_BYTES
     x = _device_payload(n, e, seed=4)
     out = torch.zeros_like(x)
@@ -149,3 +158,18 @@ def test_static_scratch_rejects_oversize_plans():
     torch.cuda.synchronize()
     assert int(out.abs().sum()) == 0  # nothing ran
     assert "static scratch" in bm.bmmc_strerror(rc)
+
+
+def test_static_scratch_one_launch_of_any_size():
+    """A general matrix that runs as one launch uses no scratch, and may be
+    larger than it."""
+    import torch
+    n, e = 22, 16  # 64 MiB > 32 MiB
+    rows, c = wl.dense_bmmc(n, 5, _inv)
+    p = bm.Plan(n, rows, c, e)
+    assert p.num_launches == 1 and p.workspace_bytes > bm.BMMC_STATIC_SCRATCH_BYTES
+    x = _device_payload(n, e, seed=4)
+    got = _static(p, x)
+    torch.cuda.synchronize()
+    bad = oracle.count_mismatch(n, rows, c, x.cpu().numpy(), got.cpu().numpy(), elem_bytes=e)
+    assert bad == 0
