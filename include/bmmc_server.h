@@ -19,10 +19,10 @@
  *      request in the calling thread, on one stream, in submission order, with
  *      no admission control and no grouping.
  *
- * Outputs and two-pass workspaces are carved out of one device arena that the
- * server allocates at creation (its only cudaMalloc); inputs stay
- * caller-owned.  The budget counts input + output + workspace bytes of every
- * request in flight.  Latency is measured from the submission (host clock)
+ * Outputs (and workspaces, where a plan is two launches) are carved out of one
+ * device arena that the server allocates at creation (its only cudaMalloc);
+ * inputs stay caller-owned.  The budget counts input + output (+ workspace)
+ * bytes of every request in flight.  Latency is measured from the submission (host clock)
  * to a CUDA event recorded after the request's last kernel (GPU clock), the
  * two clocks being aligned when the server starts.
  */

@@ -333,7 +333,10 @@ void launch_single(bmmc_server_s *s, Req *r, int si)
         if (rc == BMMC_OK) rc = complete_plan(s, r);
         if (rc == BMMC_OK) rc = bmmc::plan_launch_pass(r->plan, 1, r->ws, r->out, st);
     } else {
-        rc = bmmc_execute_ws(r->plan, r->in, r->out, r->ws, st);
+        // without a workspace of its own a request is one launch, for which
+        // bmmc_execute allocates nothing
+        rc = r->ws ? bmmc_execute_ws(r->plan, r->in, r->out, r->ws, st)
+                   : bmmc_execute(r->plan, r->in, r->out, st);
     }
     if (rc != BMMC_OK) r->status = rc;
     if (!L.ev || cudaEventRecord(L.ev, s->streams[si]) != cudaSuccess) {
@@ -603,7 +606,8 @@ int prepare(bmmc_server_s *s, Req *r, int n, const uint64_t *rows, uint64_t c, s
         }
     }
     r->array_bytes = ((size_t)1 << n) * e;
-    r->ws_bytes = bmmc_plan_workspace_bytes(r->plan);
+    // (plans of two launches only: any other never touches a workspace)
+    r->ws_bytes = r->plan->launches() == 2 ? bmmc_plan_workspace_bytes(r->plan) : 0;
     r->bytes = 2 * (uint64_t)r->array_bytes + r->ws_bytes;
     if (align_up(r->array_bytes) + align_up(r->ws_bytes) > s->arena.size()) {
         release_plan(s, r);

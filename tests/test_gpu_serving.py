@@ -89,7 +89,7 @@ def test_budget_blocks_admission():
     overlap, and all of them still finish."""
     import torch
     reqs = _requests(12, rate=1e6, n_lo=22, n_hi=22, seed=13)
-    one = max(2 * (1 << r.n) * r.e * 2 for r in reqs)
+    one = max(3 * (1 << r.n) * r.e for r in reqs)  # input and output, and half again
     srv = serving.Server("cuda", budget_bytes=one, arena_bytes=2 << 30, streams=4,
                          keep_outputs=True)
     serving.drive(srv, reqs)
@@ -221,14 +221,47 @@ def test_submit_errors():
     n = 20
     singular = [1 << i for i in range(n - 1)] + [1]
     assert srv.submit(1, n, singular, 0, 4, x) == bm.BMMC_ERR_SINGULAR
-    rows, c = wl.dense_bmmc(n, 1, _inv)  # output + workspace = 8 MiB: fits
+    rows, c = wl.dense_bmmc(n, 1, _inv)  # output = 4 MiB: fits
     assert srv.submit(2, n, rows, c, 4, x) == bm.BMMC_OK
-    big = torch.zeros(1 << 24, dtype=torch.int32, device="cuda")
-    rows24, c24 = wl.dense_bmmc(24, 1, _inv)  # 128 MiB > 64 MiB arena
-    assert srv.submit(3, 24, rows24, c24, 4, big) == bm.BMMC_ERR_TOO_LARGE
+    big = torch.zeros(1 << 25, dtype=torch.int32, device="cuda")
+    rows25, c25 = wl.dense_bmmc(25, 1, _inv)  # 128 MiB > 64 MiB arena
+    assert srv.submit(3, 25, rows25, c25, 4, big) == bm.BMMC_ERR_TOO_LARGE
     srv.drain()
     res = srv.results()
     assert [r[0] for r in res] == [2] and res[0][1] == bm.BMMC_OK
+    # the output alone is the whole arena: a general matrix has no workspace
+    rows24, c24 = wl.dense_bmmc(24, 1, _inv)
+    assert srv.submit(4, 24, rows24, c24, 4, big[: 1 << 24]) == bm.BMMC_OK
+    srv.drain()
+    res = srv.results()
+    assert [r[0] for r in res] == [4] and res[0][1] == bm.BMMC_OK
+    srv.close()
+
+
+@pytest.mark.parametrize("group_min", [0, 2])
+def test_budget_counts_input_and_output(group_min):
+    """General matrices run as one launch: a burst of them has its inputs and
+    outputs in flight, and no workspace."""
+    import torch
+    ns = [14, 16, 18, 20]
+    srv = serving.Server("cuda", budget_bytes=1 << 30, arena_bytes=1 << 30,
+                         group_min=group_min, keep_outputs=True)
+    reqs = []
+    for i, n in enumerate(ns):
+        rows, c = wl.dense_bmmc(n, 80 + n, _inv)
+        reqs.append(serving.Request(i, 0.0, n, 4, rows, c, wl.payload_torch(n, 4, seed=i)))
+    srv.hold(True)  # admitted in one round
+    for r in reqs:
+        assert srv.submit(r.rid, r.n, r.rows, r.c, r.e, r.x) == bm.BMMC_OK
+    srv.hold(False)
+    srv.drain()
+    assert srv.stats()["peak_bytes_in_flight"] == sum(2 * 4 << n for n in ns)
+    outs = {rid: (st, out) for rid, st, _, _, out in srv.results()}
+    for r in reqs:
+        st, r.out_ptr = outs[r.rid]
+        assert st == bm.BMMC_OK
+        assert torch.equal(_output(r), _solo(r, bm.BMMC_PLAN_PAPER))
+        srv.release(r.out_ptr)
     srv.close()
 
 
