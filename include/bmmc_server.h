@@ -5,9 +5,8 @@
  * thread and served on the current device.  Two modes:
  *
  *  BMMC_SERVER_CONTINUOUS  A scheduler thread admits each submitted request
- *      (planned in the submitting thread: the first pass only; the tables of
- *      a second pass are derived right after the first pass is launched,
- *      while it runs) as soon as its device bytes fit in the HBM budget, and launches it on the least-loaded of S streams, so
+ *      (planned in the submitting thread) as soon as its device bytes fit in
+ *      the HBM budget, and launches it on the least-loaded of S streams, so
  *      that requests that arrive while others run start at once and overlap
  *      with them on the device.  Small requests that are admitted together
  *      are grouped into one persistent batch launch (bmmc_batch.h).  A request
@@ -85,10 +84,9 @@ int bmmc_server_create(bmmc_server *out, const bmmc_server_config *cfg);
  * (conventions of bmmc.h; `in` is read when the request runs and must stay
  * valid until it completes).  Thread-safe.  CONTINUOUS: returns at once.
  * PLAIN: returns after planning and launching.  Errors found at submission
- * (INVALID, SINGULAR, UNSUPPORTED, TOO_LARGE for a request whose output and
- * workspace can never fit the arena) are returned here and the request is
- * not queued.  In CONTINUOUS mode a second pass is planned at launch; a
- * planning error there becomes the request's result status. */
+ * (INVALID, SINGULAR, UNSUPPORTED, TOO_LARGE for a request whose output (and
+ * workspace) can never fit the arena) are returned here and the request is
+ * not queued. */
 int bmmc_server_submit(bmmc_server s, uint64_t id, int n, const uint64_t *A_rows,
                        uint64_t c, size_t elem_bytes, const void *in);
 

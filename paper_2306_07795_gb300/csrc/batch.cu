@@ -468,7 +468,7 @@ int batch_create_impl(bmmc_batch *out, const bmmc_plan *plans, int count,
     uint64_t off = 0;
     for (int i = 0; i < count; ++i) {
         const bmmc_plan p = plans[i];
-        if (!p || !ins[i] || !outs[i] || p->derived < p->npass) return BMMC_ERR_INVALID;
+        if (!p || !ins[i] || !outs[i]) return BMMC_ERR_INVALID;
         if (((uintptr_t)ins[i] | (uintptr_t)outs[i]) & 15u) return BMMC_ERR_ALIGN;
         const uint64_t b = p->bytes();
         ranges.push_back({(uintptr_t)ins[i], (uintptr_t)ins[i] + b, false});

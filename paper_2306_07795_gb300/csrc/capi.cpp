@@ -70,7 +70,6 @@ int derive_one(bmmc_plan_s *p, int i)
 // its factors here, on first use.
 int need_passes(bmmc_plan_s *p)
 {
-    if (p->derived < p->npass) return BMMC_ERR_INVALID;
     if (!p->fused) return BMMC_OK;
     std::lock_guard<std::mutex> lock(p->derive_mu);
     for (int i = 0; i < p->npass && !p->factors_derived; ++i) {
@@ -81,10 +80,8 @@ int need_passes(bmmc_plan_s *p)
     return BMMC_OK;
 }
 
-// derive_passes: how many passes get their tables now (the rest later, by
-// plan_derive_rest).
 int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
-                size_t elem_bytes, const bmmc_plan_options *opts, int derive_passes = 2)
+                size_t elem_bytes, const bmmc_plan_options *opts)
 {
     if (!out) return BMMC_ERR_INVALID;
     *out = nullptr;
@@ -163,18 +160,14 @@ int create_impl(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
     // at most 2^(16 - e_log) bytes), so creation cannot fail for want of
     // them and only queries derive them.  Chosen segments are the caller's
     // tiles for the two passes, which then run as asked.
-    if (p->npass == 2 && opt.seg_bits == 0 &&
-        derive_tables(p, a, c, &p->whole, &p->whole_info) == 0) {
-        p->fused = true;
-        p->derived = 2;
-    }
-    for (int i = p->derived; i < p->npass && i < derive_passes; ++i) {
+    p->fused = p->npass == 2 && opt.seg_bits == 0 &&
+               derive_tables(p, a, c, &p->whole, &p->whole_info) == 0;
+    for (int i = 0; i < p->npass && !p->fused; ++i) {
         int rc = derive_one(p, i);
         if (rc) {
             delete p;
             return rc;
         }
-        p->derived = i + 1;
     }
     *out = p;
     return BMMC_OK;
@@ -186,7 +179,6 @@ int execute_impl(bmmc_plan p, const void *in, void *out, void *ws, bool takes_ws
                  cudaStream_t s, int key = 0)
 {
     const uint64_t bytes = array_bytes(p);
-    if (p->derived < p->npass) return BMMC_ERR_INVALID;
     if (((uintptr_t)in | (uintptr_t)out) & 15u) return BMMC_ERR_ALIGN;
     if (overlap(in, out, bytes)) return BMMC_ERR_ALIAS;
     if (takes_ws) {
@@ -211,39 +203,6 @@ int verify_impl(bmmc_plan p, uint64_t max_ctas);
 int describe_impl(bmmc_plan p, char *buf, size_t len);
 
 }  // namespace
-
-namespace bmmc {
-
-int plan_create_first_pass(bmmc_plan *out, int n, const uint64_t *rows, uint64_t c,
-                           size_t elem_bytes, const bmmc_plan_options *opts)
-{
-    return guarded([&] { return create_impl(out, n, rows, c, elem_bytes, opts, 1); });
-}
-
-int plan_derive_rest(bmmc_plan p)
-{
-    if (!p) return BMMC_ERR_INVALID;
-    return guarded([&] {
-        for (int i = p->derived; i < p->npass; ++i) {
-            const int rc = derive_one(p, i);
-            if (rc) return rc;
-            p->derived = i + 1;
-        }
-        return (int)BMMC_OK;
-    });
-}
-
-int plan_launch_pass(bmmc_plan p, int pass, const void *in, void *out, bmmc_stream_t s)
-{
-    if (!p || !in || !out || pass < 0 || pass >= p->derived) return BMMC_ERR_INVALID;
-    if (((uintptr_t)in | (uintptr_t)out) & 15u) return BMMC_ERR_ALIGN;
-    if (overlap(in, out, array_bytes(p))) return BMMC_ERR_ALIAS;
-    if (debug_fail_launch()) return BMMC_ERR_CUDA;
-    return launch_pass(p->desc[pass], in, out, (cudaStream_t)s, 0) == cudaSuccess ? BMMC_OK
-                                                                         : BMMC_ERR_CUDA;
-}
-
-}  // namespace bmmc
 
 extern "C" {
 

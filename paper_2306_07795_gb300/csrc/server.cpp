@@ -1,17 +1,15 @@
 // server.cpp -- native request server (include/bmmc_server.h).
 //
 // Submission plans the request in the caller's thread (bmmc_plan_create_ex),
-// so planning cost scales with the number of submitting threads; in
-// CONTINUOUS mode only the first pass is planned then, and the second pass of
-// a two-pass plan is derived right after the first pass is launched, while it
-// runs.  In CONTINUOUS mode a scheduler thread then admits requests in submission order
-// while their input + output + workspace bytes fit the budget and their output
-// and workspace fit the arena, launches each on the least-loaded stream (small
-// ones admitted together share one batch launch), and retires launches as
-// their events complete.  A request that finds nothing queued ahead of it and
-// the scheduler idle is admitted and launched in the submitting thread.  PLAIN
-// mode does planning, allocation and launch in the submitting thread on one
-// stream.  The paper has no serving counterpart (Sec. 6 times one array at a
+// so planning cost scales with the number of submitting threads.  In
+// CONTINUOUS mode a scheduler thread then admits requests in submission order
+// while their input + output (+ workspace) bytes fit the budget and their
+// output (and workspace) fits the arena, launches each on the least-loaded
+// stream (small ones admitted together share one batch launch), and retires
+// launches as their events complete.  A request that finds nothing queued
+// ahead of it and the scheduler idle is admitted and launched in the submitting
+// thread.  PLAIN mode does planning, allocation and launch in the submitting
+// thread on one stream.  The paper has no serving counterpart (Sec. 6 times one array at a
 // time); every request runs the passes of Sec. 5.1 / 5.2 unchanged.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -313,11 +311,6 @@ void note_peaks(bmmc_server_s *s)
     s->peak_inflight = std::max<uint64_t>(s->peak_inflight, s->n_inflight);
 }
 
-// Derive the tables a request's plan still lacks (sched_mu held: every
-// launch, and so every completion of a plan, even a cached one shared by
-// several requests, happens under it).
-int complete_plan(bmmc_server_s *, Req *r) { return bmmc::plan_derive_rest(r->plan); }
-
 // Launch one request on stream si (sched_mu held, buffers allocated).  A
 // request that fails to launch still completes, with its error status, once
 // the stream reaches its event.
@@ -326,18 +319,10 @@ void launch_single(bmmc_server_s *s, Req *r, int si)
     Launch L;
     L.ev = take_event(s);
     const bmmc_stream_t st = (bmmc_stream_t)s->streams[si];
-    int rc;
-    if (r->plan->derived < r->plan->npass) {
-        // The first pass runs while the host derives the second pass's tables.
-        rc = bmmc::plan_launch_pass(r->plan, 0, r->in, r->ws, st);
-        if (rc == BMMC_OK) rc = complete_plan(s, r);
-        if (rc == BMMC_OK) rc = bmmc::plan_launch_pass(r->plan, 1, r->ws, r->out, st);
-    } else {
-        // without a workspace of its own a request is one launch, for which
-        // bmmc_execute allocates nothing
-        rc = r->ws ? bmmc_execute_ws(r->plan, r->in, r->out, r->ws, st)
-                   : bmmc_execute(r->plan, r->in, r->out, st);
-    }
+    // without a workspace of its own a request is one launch, for which
+    // bmmc_execute allocates nothing
+    const int rc = r->ws ? bmmc_execute_ws(r->plan, r->in, r->out, r->ws, st)
+                         : bmmc_execute(r->plan, r->in, r->out, st);
     if (rc != BMMC_OK) r->status = rc;
     if (!L.ev || cudaEventRecord(L.ev, s->streams[si]) != cudaSuccess) {
         // no event: wait here so that completion is known
@@ -359,8 +344,6 @@ bool launch_group(bmmc_server_s *s, std::vector<Req *> &g, int si)
     std::vector<bmmc_plan> plans;
     std::vector<const void *> ins;
     std::vector<void *> outs;
-    for (Req *r : g)  // a batch takes complete plans only
-        if (complete_plan(s, r) != BMMC_OK) return false;
     for (Req *r : g) {
         plans.push_back(r->plan);
         ins.push_back(r->in);
@@ -586,11 +569,7 @@ int prepare(bmmc_server_s *s, Req *r, int n, const uint64_t *rows, uint64_t c, s
         memset(&o, 0, sizeof(o));
         o.flags = s->cfg.plan_flags;
         bmmc_plan p = nullptr;
-        // Continuous mode plans the first pass only: the second pass's tables
-        // are derived at launch, while the first pass runs.
-        const bool staged = s->cfg.mode == BMMC_SERVER_CONTINUOUS;
-        int rc = staged ? bmmc::plan_create_first_pass(&p, n, rows, c, e, &o)
-                        : bmmc_plan_create_ex(&p, n, rows, c, e, &o);
+        const int rc = bmmc_plan_create_ex(&p, n, rows, c, e, &o);
         if (rc != BMMC_OK) return rc;
         r->plan = p;
         if (use_cache) {
