@@ -98,8 +98,8 @@ struct SortDesc {
 };
 
 // The whole network on one thread block, for arrays of at most 2^7 keys: the
-// keys stay in shared memory at their virtual positions, and the block writes
-// key x to out[fin x] at the end.
+// keys stay in shared memory at their virtual positions, which are also where
+// the network leaves them.
 struct SortSmallDesc {
     uint32_t N;        // 2^N keys
     uint32_t key;
@@ -107,7 +107,6 @@ struct SortSmallDesc {
     uint32_t pad;
     uint32_t u[kSortSmallMaxStages];
     uint32_t g[kSortSmallMaxStages];
-    uint32_t fin[kSortSmallMaxBits];  // row masks of the final layout
 };
 
 }  // namespace bmmc

@@ -2,16 +2,16 @@
 //
 // A fused pass is the tiled BMMC pass of Sec. 4.1 (16-byte asynchronous copies
 // into swizzled shared memory, barrier, 16-byte gathers and stores) with
-// comparator stages run on the tile in between.  The stages come in groups (sort_desc.h): for one group, every
-// thread loads 2^R keys of the tile into registers, and each stage of the group
-// orders pairs of those registers, the pair's low position (index with
-// g_s . x = 0) receiving the smaller key (Sec. 6.1: a pair is kept when
-// first <= second and swapped otherwise).  The keys go back to the same slots,
-// and a barrier separates the groups.
+// comparator stages run on the tile in between.  The stages come in groups
+// (sort_desc.h): for one group, every thread loads 2^R keys of the tile into
+// registers, and each stage of the group orders pairs of those registers, the
+// pair's low position (index with g_s . x = 0) receiving the smaller key
+// (Sec. 6.1: a pair is kept when first <= second and swapped otherwise).  The
+// keys go back to the same slots, and a barrier separates the groups.
 //
 // Arrays of at most 2^12 keys are one block of that kernel; those of at most
 // 2^7 run in bmmc_sort_small: keys at their positions in shared memory, one
-// stage at a time, then each key to its final position.
+// stage at a time.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(256)
         __syncthreads();
     }
     for (uint32_t x = threadIdx.x; x < count; x += blockDim.x)
-        dst[bmmc_map(d.fin, d.N, 0u, x)] = sm[x];
+        dst[x] = sm[x];
 }
 
 template <typename... Args>

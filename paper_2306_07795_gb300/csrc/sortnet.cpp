@@ -817,7 +817,6 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
             U.push_back((1ull << (n - i)) - (1ull << (n - l)));
             G.push_back(1ull << (n - 1 - i));
         }
-    const f2::Mat qfin = f2::Mat::identity(N);
 
     if (N <= kSortSmallMaxBits) {
         SortSmallDesc &d = p->sdesc;
@@ -829,7 +828,6 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
             d.u[s] = (uint32_t)U[s];
             d.g[s] = (uint32_t)G[s];
         }
-        for (int i = 0; i < N; ++i) d.fin[i] = (uint32_t)qfin.r[i];
         p->small = true;
         return BMMC_OK;
     }
@@ -879,7 +877,7 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
         for (int attempt = 0; attempt < (last ? 1 : kTries) && best != 0; ++attempt) {
             f2::Mat L, L_inv;
             if (last) {
-                L = L_inv = qfin;
+                L = L_inv = f2::Mat::identity(N);
             } else {
                 std::vector<uint64_t> cols = pp.out;
                 Span sp;
@@ -990,12 +988,7 @@ int emulate(const bmmc_sort_plan_s *p, const void *in_v, void *out_v)
                 if (__builtin_parityll(x & d.g[s]) != 0) continue;  // x is the low one
                 order_pair(p->key, &a[x], &a[y]);
             }
-        for (uint64_t x = 0; x < count; ++x) {
-            uint64_t y = 0;
-            for (uint32_t i = 0; i < d.N; ++i)
-                y |= (uint64_t)__builtin_parityll(d.fin[i] & x) << i;
-            store_key(out, y, e_log, a[x]);
-        }
+        for (uint64_t x = 0; x < count; ++x) store_key(out, x, e_log, a[x]);
         return 0;
     }
     std::vector<uint8_t> bufs[2];
