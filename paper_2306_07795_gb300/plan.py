@@ -137,8 +137,10 @@ class Plan:
         dev = x.get_device()
         raw = stream.cuda_stream if stream is not None else current_raw_stream(dev)
         if workspace is None and self._direct is not None:
+            name = "bmmc_execute_direct"
             code = on_device(dev, self._direct, self._h, x.data_ptr(), out.data_ptr(), 1, raw)
         else:
+            name = "bmmc_execute_ws"
             ws_bytes = self._ws_bytes
             if ws_bytes is None:
                 ws_bytes = self._ws_bytes = self.workspace_bytes
@@ -148,7 +150,7 @@ class Plan:
             code = on_device(dev, B.lib().bmmc_execute_ws, self._h, x.data_ptr(),
                              out.data_ptr(), ws_ptr, raw)
         if code != B.BMMC_OK:
-            raise B.BmmcError(code, "bmmc_execute_ws")
+            raise B.BmmcError(code, name)
         return out
 
     def run_rows(self, x, rows):

@@ -70,6 +70,17 @@ def test_one_launch_allocates_no_workspace():
         assert np.array_equal(y.cpu().numpy().view(np.uint32), want)
 
 
+def test_errors_name_the_entry_point():
+    import torch
+    n, e, rows, c = _dense()
+    x = torch.arange(1 << n, dtype=torch.int32, device="cuda")
+    for seg_bits, name in ((0, "bmmc_execute_direct"), (6, "bmmc_execute_ws")):
+        p = bm.Plan(n, rows, c, e, seg_bits=seg_bits)
+        bm.bmmc_debug_fail_launches(1)
+        with pytest.raises(bm.BmmcError, match=name + " failed"):
+            p(x)
+
+
 @pytest.mark.parametrize("passes", [1, 2])
 def test_launch_failure(passes):
     import torch
