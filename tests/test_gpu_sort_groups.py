@@ -1,8 +1,11 @@
 """The register groups of the fused sorting passes at their edges: one block and
 the first sizes beyond, every count of keys per thread, and float keys that are
-all ordinary or hold a single NaN or a single -0.0 (one thread block then
-compares with IEEE <=, the others by minimum and maximum or as integers).  Bit
-for bit the host emulation of the same plan."""
+all ordinary or hold a single special one (the thread block with it then
+compares as IEEE <=, the others by minimum and maximum or as integers).  The
+kernel looks for special keys by the extremes of their bits, so NaN of either
+sign and -0.0 come alone, and for doubles also what the high word cannot tell
+from them: infinities and the smallest negative numbers.  Bit for bit the host
+emulation of the same plan."""
 
 import ctypes
 
@@ -29,16 +32,35 @@ def _keys(dtype, count, special, seed):
     x[g.integers(0, count, 8)] = 0.0
     x[g.integers(0, count, 4)] = np.finfo(dtype).smallest_subnormal
     x[g.integers(0, count, 4)] = -np.finfo(dtype).max
-    x[g.integers(0, count)] = np.inf
+    if dtype == np.float32:  # ordinary keys in 4 bytes
+        x[g.integers(0, count, 2)] = np.inf
+        x[g.integers(0, count, 2)] = -np.inf
+        x[g.integers(0, count, 2)] = -np.finfo(dtype).smallest_subnormal
     if special is not None:
         x[g.integers(0, count)] = special
     return x
 
 
-@pytest.mark.parametrize("dtype,special", [(np.float32, None), (np.float32, np.nan),
-                                           (np.float32, -0.0), (np.float64, None),
-                                           (np.float64, np.nan), (np.float64, -0.0),
-                                           (np.int32, None), (np.uint64, None)])
+SPECIAL = [np.nan, np.copysign(np.nan, -1.0), -0.0]
+SPECIAL64 = SPECIAL + [np.inf, -np.inf, -np.finfo(np.float64).smallest_subnormal]
+
+
+def test_keys_are_as_ordinary_as_they_say():
+    """What the kernel takes for special, restated: no key without `special`,
+    one with."""
+    for dtype, special in [(np.float32, v) for v in [None] + SPECIAL] + \
+            [(np.float64, v) for v in [None] + SPECIAL64]:
+        x = _keys(dtype, 1 << 8, special, 1)
+        odd = np.isnan(x) | ((x == 0) & np.signbit(x))
+        if dtype == np.float64:
+            odd |= np.isinf(x) | ((x < 0) & (x > -2.0 ** -1042))
+        assert odd.sum() == (0 if special is None else 1)
+
+
+@pytest.mark.parametrize("dtype,special", [(np.float32, None)] +
+                         [(np.float32, v) for v in SPECIAL] + [(np.float64, None)] +
+                         [(np.float64, v) for v in SPECIAL64] +
+                         [(np.int32, None), (np.uint64, None)])
 @pytest.mark.parametrize("n,b,block_log2", [(7, 0, 0), (8, 0, 0), (9, 0, 0), (11, 0, 0), (12, 0, 0),
                                             (13, 0, 0), (13, 0, 16), (14, 0, 16), (15, 1, 15),
                                             (8, 6, 0), (20, 0, 0)])
