@@ -20,11 +20,14 @@ extern "C" {
  * BMMC_ERR_OOM.  count <= 0 clears the counter. */
 void bmmc_debug_fail_allocs(int count);
 
-/* The next `count` launches (one per pass of bmmc_execute*, one per phase
- * launch of a batch) are not made and report a launch failure: the entry
+/* The next `count` launches (one or two of bmmc_execute*, one per phase
+ * launch of a batch, one per pass of a sort) are not made and report a launch failure: the entry
  * point returns BMMC_ERR_CUDA (a server records it as the request's
  * status).  count <= 0 clears the counter. */
 void bmmc_debug_fail_launches(int count);
+
+/* The same for the `count` launches after the next `after`, which are made. */
+void bmmc_debug_fail_launches_after(int after, int count);
 
 #ifdef __cplusplus
 }

@@ -81,24 +81,27 @@ def test_errors_name_the_entry_point():
             p(x)
 
 
-@pytest.mark.parametrize("passes", [1, 2])
-def test_launch_failure(passes):
+@pytest.mark.parametrize("passes,seg_bits,launches,failing", [(1, 0, 1, 0), (2, 0, 1, 0),
+                                                              (2, 6, 2, 0), (2, 6, 2, 1)])
+def test_launch_failure(passes, seg_bits, launches, failing):
+    """The launch `failing` of a plan fails (the first ones run)."""
     import torch
     n, e = 18, 4
     if passes == 2:
         rows, c = wl.dense_bmmc(n, 3, _inv)
     else:
         rows, c = wl.bit_reverse(n), 5
-    p = bm.Plan(n, rows, c, e)
-    assert p.num_passes == passes
+    p = bm.Plan(n, rows, c, e, seg_bits=seg_bits)
+    assert (p.num_passes, p.num_launches) == (passes, launches)
     x = torch.arange(1 << n, dtype=torch.int32, device="cuda")
-    y = torch.empty_like(x)
+    y = torch.full_like(x, -1)
     ws = torch.empty(max(p.workspace_bytes, 16), dtype=torch.uint8, device="cuda")
     s = torch.cuda.current_stream().cuda_stream
-    bm.bmmc_debug_fail_launches(1)
+    bm.bmmc_debug_fail_launches_after(failing, 1)
     with pytest.raises(bm.BmmcError) as ei:
         bm.bmmc_execute_ws(p.handle, x.data_ptr(), y.data_ptr(), ws.data_ptr(), s)
     assert ei.value.code == bm.BMMC_ERR_CUDA
+    assert bool((y == -1).all())  # the launch that writes y was not made
     # the failure is consumed: the next call runs
     y2 = p(x, workspace=ws)
     torch.cuda.synchronize()

@@ -187,7 +187,9 @@ def test_execute_host_buffers(e):
     streams = [torch.cuda.Stream() for _ in range(3)]
     jobs = []
     for i, (name, rows, c) in enumerate(cases):
-        p = bm.Plan(n, rows, c, e)
+        # chosen segments, and so two launches, for the last ones
+        p = bm.Plan(n, rows, c, e, seg_bits=8 - (e.bit_length() - 1) if i >= 3 else 0)
+        assert p.num_launches == (2 if i >= 3 else 1)
         pinned = i % 2 == 0
         h_in = torch.from_numpy(flat.copy())
         h_out = torch.zeros_like(h_in)
@@ -227,13 +229,17 @@ def test_execute_host_errors():
     torch.cuda.synchronize()
 
 
-def test_concurrent_streams_distinct_workspaces():
+@pytest.mark.parametrize("seg_bits,launches", [(0, 1), (6, 2)])
+def test_concurrent_streams_distinct_workspaces(seg_bits, launches):
+    """Calls in flight on four streams: as one launch, and as two through a
+    workspace each."""
     import torch
     n = 20
     plans, xs = [], []
     for s in range(4):
         rows, c = wl.dense_bmmc(n, 50 + s, oracle_invertible)
-        plans.append(bm.Plan(n, rows, c, 4))
+        plans.append(bm.Plan(n, rows, c, 4, seg_bits=seg_bits))
+        assert plans[-1].num_launches == launches
         xs.append(to_device(wl.payload(n, 4, seed=s)))
     want = [p(x) for p, x in zip(plans, xs)]
     torch.cuda.synchronize()

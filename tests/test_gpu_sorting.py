@@ -48,15 +48,18 @@ def _values(np_dtype, count, seed):
 
 
 @pytest.mark.parametrize("name,key,np_dtype", KEYS)
-@pytest.mark.parametrize("flags", [bm.BMMC_PLAN_PAPER, bm.BMMC_PLAN_SINGLE_PASS])
-def test_execute_ce_matches_reference(name, key, np_dtype, flags):
+@pytest.mark.parametrize("flags,two", [(bm.BMMC_PLAN_PAPER, False), (bm.BMMC_PLAN_PAPER, True),
+                                       (bm.BMMC_PLAN_SINGLE_PASS, False)])
+def test_execute_ce_matches_reference(name, key, np_dtype, flags, two):
+    """two: chosen segments, so that the comparators follow a second launch."""
     import torch
     e = np.dtype(np_dtype).itemsize
     for n in (3, 6, 9, 14, 19):
         rows, c = wl.dense_bmmc(n, 30 + n, _inv)
         arr = _values(np_dtype, 1 << n, n)
         want = _ce_ref(oracle.apply(n, rows, c, arr, elem_bytes=e))
-        p = bm.Plan(n, rows, c, e, flags=flags)
+        p = bm.Plan(n, rows, c, e, flags=flags, seg_bits=8 - (e.bit_length() - 1) if two else 0)
+        assert p.num_launches == (2 if two and e << n > 1 << 16 else 1)
         x = torch.from_numpy(arr.view(np.int32 if e == 4 else np.int64).copy()).cuda()
         y = torch.empty_like(x)
         ws = torch.empty(max(p.workspace_bytes, 16), dtype=torch.uint8, device="cuda")
@@ -130,15 +133,18 @@ def test_execute_ce_full_size(name, key, np_dtype):
     arr = _values(np_dtype, 1 << n, 11)
     want = _ce_ref(oracle.apply(n, rows, c, arr, elem_bytes=e))
     x = torch.from_numpy(arr.view(np.int32 if e == 4 else np.int64).copy()).cuda()
-    for flags in (bm.BMMC_PLAN_PAPER, bm.BMMC_PLAN_SINGLE_PASS):
-        p = bm.Plan(n, rows, c, e, flags=flags)
+    for flags, seg_bits, launches in ((bm.BMMC_PLAN_PAPER, 0, 1),
+                                      (bm.BMMC_PLAN_PAPER, 8 - (e.bit_length() - 1), 2),
+                                      (bm.BMMC_PLAN_SINGLE_PASS, 0, 1)):
+        p = bm.Plan(n, rows, c, e, flags=flags, seg_bits=seg_bits)
+        assert p.num_launches == launches
         y = torch.empty_like(x)
         ws = torch.empty(max(p.workspace_bytes, 16), dtype=torch.uint8, device="cuda")
         bm.bmmc_execute_ce(p.handle, x.data_ptr(), y.data_ptr(), ws.data_ptr(), key,
                            torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         got = y.cpu().numpy().view(np_dtype)
-        assert np.array_equal(got.view(np.uint8), want.view(np.uint8)), (name, flags)
+        assert np.array_equal(got.view(np.uint8), want.view(np.uint8)), (name, flags, seg_bits)
         del y, ws
 
 
