@@ -7,25 +7,34 @@ two tiled passes (Sec. 4), all done on the host by the C library."""
 from . import _binding as B
 
 
-_raw_stream_getter = None
+_raw = None
+
+
+def _raw_accessors():
+    """PyTorch's raw accessors, looked up once: the current stream of a CUDA device
+    and the current device.  The Stream object they skip is 2 us of a call, the
+    checked form of the second 0.2 us (whoever holds a CUDA tensor has CUDA
+    initialised)."""
+    global _raw
+    if _raw is None:
+        import torch
+        _raw = (getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+                    lambda i: torch.cuda.current_stream(i).cuda_stream),
+                getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device)
+    return _raw
 
 
 def current_raw_stream(index):
     """The cudaStream_t of PyTorch's current stream on CUDA device `index`, as an
-    int.  The raw accessor skips building a Stream object (2 us of a call)."""
-    global _raw_stream_getter
-    if _raw_stream_getter is None:
-        import torch
-        _raw_stream_getter = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
-            lambda i: torch.cuda.current_stream(i).cuda_stream)
-    return _raw_stream_getter(index)
+    int."""
+    return (_raw or _raw_accessors())[0](index)
 
 
 def on_device(index, fn, *args):
     """fn(*args) with CUDA device `index` current; returns its result."""
-    import torch
-    if index == torch.cuda.current_device():
+    if index == (_raw or _raw_accessors())[1]():
         return fn(*args)
+    import torch
     with torch.cuda.device(index):
         return fn(*args)
 
