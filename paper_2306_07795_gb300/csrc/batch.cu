@@ -293,15 +293,19 @@ cudaError_t prepare_group(Group *g, int sms)
     uint64_t grid = (uint64_t)sms * (uint64_t)per_sm;
     if (grid > g->total) grid = g->total;
     g->grid = (uint32_t)grid;
-    // Chunks of about 1/64 of a block's share of the items: the blocks resident
-    // at a time then work on nearby tiles, and the launch ends evenly; at least
-    // 8 items, since a chunk costs a search and often a table, and 4 where a
-    // block's share is a few such chunks, which 8 would split unevenly.
-    // (Chunks of 16 / 8 / 4 items: 1024 arrays of 2^10..2^20, share 70: 240 / 231 /
-    // 235 us; 200 arrays of 2^12..2^18, share 12: 48 / 61 / 47 us.)
+    // A chunk costs a search and often a table, and chunks that do not divide a
+    // block's share leave some blocks one more than the others; many small ones
+    // keep the blocks that run at a time on nearby tiles and end the launch
+    // evenly.  So: the whole share of up to 12 items, 4 items up to a share of
+    // 48, from there 8, or 1/64 of the share where that is more.  Measured, us
+    // with chunks of 4 / 8 / the whole share, 4-byte arrays of 2^12..2^18: share
+    // 5: 32 / 24 / 24, 10: 45 / 59 / 45, 14: 58 / 68 / 57, 18: 70 / 77 / 71,
+    // 26: 92 / 99 / 98, 39: 133 / 134 / 139, 48: 164 / 162 / 173, 101: 329 /
+    // 315 / - (16: 321); within 3 % of these ratios for 8-byte arrays of the
+    // same sizes, 2^10..2^16 and 2^14..2^20.
     const uint64_t per = (g->total + grid - 1) / grid;
     uint64_t chunk = per / 64;
-    if (chunk < 8) chunk = per < 32 ? 4 : 8;
+    if (chunk < 8) chunk = per <= 12 ? per : per < 48 ? 4 : 8;
     if (chunk > per) chunk = per;
     g->chunk = (uint32_t)chunk;
     return cudaSuccess;
