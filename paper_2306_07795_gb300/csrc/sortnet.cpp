@@ -841,7 +841,11 @@ int plan_sort(bmmc_sort_plan_s *p, int n, int b, int key, int block_log2)
     // starts to win (GB300, us, 2^12 / 2^13 / 2^14 4-byte keys: n = 18 float32
     // 35 / 49 / 72, n = 20 66 / 64 / 95, n = 23 444 / 361 / 381, n = 24
     // 984 / 805 / 721; 2^12 / 2^13 8-byte keys: n = 22 int64 355 / 383,
-    // n = 23 810 / 731).
+    // n = 23 810 / 731).  They hold for rows too, also where a larger block would
+    // keep whole rows and so be one pass (float32, 2^12 / 2^13 / 2^14 keys a
+    // block: 64 rows of 2^13 18.6 / 24.8 / 43.1, 512 rows of 2^13 63.9 / 72.4 /
+    // 73.8, 512 rows of 2^14 142 / 115 / 180; int64, 2^12 / 2^13: 512 rows of
+    // 2^13 114 / 125, 1024 rows 227 / 215).
     int D = block_log2 ? block_log2 - e_log : kMinBlockBits;
     if (!block_log2)
         D += e_log == 2 ? (N >= 20) + (N >= 24) : (N >= 23);
