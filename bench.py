@@ -279,6 +279,10 @@ def profiled_traffic(kernel_name):
         return None, None
 
 
+# What the strategies run: with the default segments every matrix is one launch.
+STRATEGY = {"paper": "paper, two-pass plans as one launch", "single": "single"}
+
+
 def workload_config(args, world):
     """The `config` object of both arms' JSON lines (the same workload)."""
     elems = [int(v) for v in args.elem.split(",")]
@@ -288,7 +292,7 @@ def workload_config(args, world):
         "workload": "n=%d BMMC permutation set per elem size: bit-reversal, "
                     "half-swap, %d random BP, %d random tiled-only, %d random "
                     "dense (random c)" % (args.n, args.bp, args.tiled, args.dense),
-        "n": args.n, "elem_bytes": elems, "strategy": args.strategy,
+        "n": args.n, "elem_bytes": elems, "strategy": STRATEGY[args.strategy],
         "tile_load": "tensor copies (TMA)" if args.load == "tma" else "16-byte cp.async",
         "permutations_per_step": count,
         "l2": "inputs larger than L2 (%d-%d MiB per array), no flush"
@@ -747,7 +751,7 @@ def bench_serving(dev, seconds=10.0, rate=2000.0, seed=11, budget=40 * 10**9, st
 
     import paper_2306_07795_gb300 as bm
     res = {"requests": len(specs), "rate_per_s": rate, "seconds": seconds,
-           "budget_bytes": budget, "streams": streams, "strategy": "paper",
+           "budget_bytes": budget, "streams": streams, "strategy": STRATEGY["paper"],
            "server_large_log2": 28}
     # The latency floor with no queueing: each request's HBM traffic (2 N e
     # per launch) at the measured peak; its 99th percentile bounds p99 from
